@@ -367,7 +367,7 @@ class _Wilson:
 
 
 def _dots(a, b):
-    return (a.conj() * b).sum(dim=tuple(range(6)))
+    return (a.conj() * b).sum(dim=tuple(range(6)), dtype=torch.complex128)
 
 
 def _solve64(M, b, dagger=False):
@@ -384,19 +384,19 @@ def _solve64(M, b, dagger=False):
         if float((nrm / b2.sqrt()).max()) < 1e-13:
             break
         r = (r64 / nrm.clamp_min(1e-300)).to(torch.complex64)
-        e, rh, p = torch.zeros_like(r), r.clone(), r.clone()
+        e, rh, p = torch.zeros_like(r), m(m(r)), r.clone()  # (a point source is its own shadow's breakdown)
         rho = _dots(rh, r)
         for it in range(600):
             v = m(p)
             on = _dots(r, r).real > 1e-11  # a column that is done stays as it is
-            al = torch.where(on, rho / _dots(rh, v), 0)
+            al = torch.where(on, rho / _dots(rh, v), 0).to(r.dtype)
             s = r - al * v
             t = m(s)
-            om = torch.where(on, _dots(t, s) / _dots(t, t).real.clamp_min(1e-30), 0)
+            om = torch.where(on, _dots(t, s) / _dots(t, t).real.clamp_min(1e-30), 0).to(r.dtype)
             e += al * p + om * s
             r = s - om * t
             new = _dots(rh, r)
-            p = r + torch.where(on, (new / rho) * (al / om), 0) * (p - om * v)
+            p = r + torch.where(on, (new / rho) * (al / om), 0).to(r.dtype) * (p - om * v)
             rho = torch.where(on, new, rho)
             if it % 4 == 3 and float(_dots(r, r).real.max()) < 1e-9:
                 break
