@@ -54,92 +54,86 @@ struct OuterState {
     int scale_exp;    // the batch's fields carry the exact factor 2^scale_exp (float-float outer loop)
 };
 
-__device__ __forceinline__ bool finite2(double2 z) { return isfinite(z.x) && isfinite(z.y); }
-__device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
-    const double d = b.x * b.x + b.y * b.y;
-    return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
+// (by the exponent bits: a comparison would be one more FP64 instruction)
+__device__ __forceinline__ bool finite1(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool finite2(double2 z) { return finite1(z.x) && finite1(z.y); }
+// 1/x by the hardware's approximation and two Newton steps.  On GB300 an FP64
+// instruction of a warp takes about 70 cycles, whatever its lanes do, and an
+// IEEE division 750 to 1500 (measured: 8 dependent divisions 12,400 cycles, 8 of
+// these reciprocals 3,100); the scalar recurrences below sit on every iteration's
+// critical path.
+__device__ __forceinline__ double fp64_rcp(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = ::fma(r, ::fma(-x, r, 1.0), r);
+    return ::fma(r, ::fma(-x, r, 1.0), r);
+}
+// a / b for b2 = |b|^2
+__device__ __forceinline__ double2 cdiv_by(double2 a, double2 b, double b2) {
+    const double i = fp64_rcp(b2);
+    return make_double2((a.x * b.x + a.y * b.y) * i, (a.y * b.x - a.x * b.y) * i);
 }
 __device__ __forceinline__ double2 cmul2(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// Sum partials[b][rhs][k] over blocks b for one right-hand side, by the whole
-// thread block (a multiple of 32 threads), in a fixed order: strided per-thread
-// sums, then warp shuffles, then the warps in index order.  Every thread gets
-// the total.
-__device__ __forceinline__ double2 sum_partials(const double2 *partials, int nblocks, int N, int NV, int rhs, int k) {
-    __shared__ double2 wsum[32];
-    double re = 0.0, im = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-        const double2 v = partials[((size_t)b * N + rhs) * NV + k];
-        re += v.x;
-        im += v.y;
-    }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-        re += __shfl_xor_sync(0xffffffffu, re, off);
-        im += __shfl_xor_sync(0xffffffffu, im, off);
-    }
-    const int nw = blockDim.x >> 5;
-    if (nw == 1) return make_double2(re, im);
-    __syncthreads();  // an earlier call may still be reading wsum
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = make_double2(re, im);
-    __syncthreads();
-    re = 0.0;
-    im = 0.0;
-    for (int w = 0; w < nw; ++w) {
-        re += wsum[w].x;
-        im += wsum[w].y;
-    }
-    return make_double2(re, im);
-}
-
-// All NV values of right-hand side `rhs` at once, each summed in exactly the
-// order of sum_partials (so the results are bitwise the same), in one pass over
-// the blocks: a thread reads the NV contiguous values of each of its blocks.
+// Sum the NV values partials[b][rhs][0 .. NV) over blocks b for one right-hand
+// side, by the whole thread block (kScalarThreads threads), in a fixed order:
+// strided per-thread sums, lanes, warps.  out[] is valid in thread 0 only.
+// FP64 additions are what this costs (a warp's takes 17 to 70 cycles): the
+// lanes exchange halves of their 2 NV values instead of each reducing all of
+// them (12 additions a warp for NV = 5 instead of 50), warps without a block
+// to read drop out, and one lane per value adds the warps.  With the divisions
+// of the scalar steps this took scalar_omega_kernel from 14.3 to 4.5 us
+// on 64 blocks.
 template <int NV>
-__device__ __forceinline__ void sum_partials_all(const double2 *partials, int nblocks, int N, int rhs,
-                                                 double2 (&out)[NV]) {
-    __shared__ double2 wsum[32][NV];
-    double re[NV], im[NV];
+__device__ __forceinline__ void sum_partials(const double2 *partials, int nblocks, int N, int rhs, double2 (&out)[NV]) {
+    constexpr int W = 2 * NV;
+    __shared__ double wsum[32][W];
+    const int lane = threadIdx.x & 31, nw = min((int)blockDim.x, (nblocks + 31) & ~31) >> 5;
+    __syncthreads();  // an earlier call may still be reading wsum
+    if ((int)(threadIdx.x >> 5) < nw) {
+        double v[W];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) re[k] = im[k] = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-        const double2 *p = partials + ((size_t)b * N + rhs) * NV;
+        for (int k = 0; k < W; ++k) v[k] = 0.0;
+        for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
+            const double2 *p = partials + ((size_t)b * N + rhs) * NV;
 #pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            const double2 v = p[k];
-            re[k] += v.x;
-            im[k] += v.y;
+            for (int k = 0; k < NV; ++k) {
+                const double2 q = p[k];
+                v[2 * k] += q.x;
+                v[2 * k + 1] += q.y;
+            }
         }
-    }
-#pragma unroll
-    for (int k = 0; k < NV; ++k)
+        int idx = 0, end = W, n = W;  // this lane still holds values idx .. end - 1, in v[0 .. n)
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1) {
-            re[k] += __shfl_xor_sync(0xffffffffu, re[k], off);
-            im[k] += __shfl_xor_sync(0xffffffffu, im[k], off);
+            const int h = (n + 1) / 2;  // (compile-time after unrolling)
+            if (n > 1) {
+                const bool up = (lane & off) != 0;  // keeps the upper part
+#pragma unroll
+                for (int k = 0; k < W / 2 + 1; ++k) {
+                    if (k >= h) break;
+                    const double lo = v[k], hi = h + k < n ? v[h + k] : 0.0;
+                    v[k] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, off);
+                }
+                if (up) idx += h;
+                else end = min(end, idx + h);
+                n = h;
+            } else {
+                v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+            }
         }
-    const int nw = blockDim.x >> 5;
-    if (nw == 1) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) out[k] = make_double2(re[k], im[k]);
-        return;
-    }
-    __syncthreads();  // an earlier call may still be reading wsum
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) wsum[threadIdx.x >> 5][k] = make_double2(re[k], im[k]);
+        if (idx < end) wsum[threadIdx.x >> 5][idx] = v[0];
     }
     __syncthreads();
+    if (threadIdx.x < 32) {
+        double t = 0.0;
+        if (lane < W)
+            for (int w = 0; w < nw; ++w) t += wsum[w][lane];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        double sr = 0.0, si = 0.0;
-        for (int w = 0; w < nw; ++w) {
-            sr += wsum[w][k].x;
-            si += wsum[w][k].y;
-        }
-        out[k] = make_double2(sr, si);
+        for (int k = 0; k < NV; ++k)
+            out[k] = make_double2(__shfl_sync(0xffffffffu, t, 2 * k), __shfl_sync(0xffffffffu, t, 2 * k + 1));
     }
 }
 
@@ -156,51 +150,53 @@ __device__ __forceinline__ double inner_reduction(const OuterState &o, double de
 }
 
 // ---------------------------------------------------------------------------
-// scalar kernels: grid = N blocks of kScalarThreads (one block per right-hand side)
+// Scalar recurrences of one right-hand side, shared by the scalar kernels below
+// and the cluster-resident solver (resident.cuh).
 // ---------------------------------------------------------------------------
-
-// Start an inner phase: rho = <rhat, r_l>, r2 = |r_l|^2 (from the partials of
-// inner_init_kernel), target and caps; records the scale sigma = |r64| of the
-// phase.  max_iters caps this phase; max_total the iterations over all phases.
-static __global__ void inner_start_kernel(RhsState *st, OuterState *os, const double2 *partials,
-                                   int nblocks, int N, double delta, int max_iters, int max_total, int fixed) {
-    const int r = blockIdx.x;
-    double2 v[2];
-    sum_partials_all<2>(partials, nblocks, N, r, v);
-    const double2 rho = v[0], n2 = v[1];
-    if (threadIdx.x != 0) return;
-    os[r].sigma = os[r].active ? sqrt(os[r].r2) : 0.0;
+__device__ __forceinline__ RhsState begin_state(OuterState &o, double r2, double delta, int max_iters, int max_total,
+                                                int fixed) {
+    o.sigma = o.active ? sqrt(o.r2) : 0.0;
     RhsState s;
-    s.rho = rho;
-    s.alpha = make_double2(1.0, 0.0);
     s.omega = make_double2(1.0, 0.0);
     s.beta = make_double2(0.0, 0.0);
-    s.r2 = n2.x;
-    s.r2_0 = n2.x;
-    const double red = inner_reduction(os[r], delta);
-    s.target2 = red * red * n2.x;
+    s.r2 = r2;
+    s.r2_0 = r2;
+    const double red = inner_reduction(o, delta);
+    s.target2 = red * red * r2;
     s.iters = 0;
     s.status = ST_OK;
-    const int left = max_total - os[r].iters;
+    const int left = max_total - o.iters;
     s.max_iters = fixed ? max_iters : (max_iters < left ? max_iters : left);
     s.fixed = fixed;
-    const bool on = os[r].active && n2.x > 0.0 && isfinite(n2.x) && (rho.x != 0.0 || rho.y != 0.0) &&
-                    s.max_iters > 0;
+    return s;
+}
+__device__ __forceinline__ RhsState bicg_begin(OuterState &o, double2 rho, double r2, double delta, int max_iters,
+                                               int max_total, int fixed) {
+    RhsState s = begin_state(o, r2, delta, max_iters, max_total, fixed);
+    s.rho = rho;
+    s.alpha = make_double2(1.0, 0.0);
+    const bool on = o.active && r2 > 0.0 && isfinite(r2) && (rho.x != 0.0 || rho.y != 0.0) && s.max_iters > 0;
     s.active = on;
     s.next_active = on;
-    st[r] = s;
+    return s;
 }
-
-// After v = Mhat p: alpha = rho / <rhat, v>.
-static __global__ void scalar_alpha_kernel(RhsState *st, const double2 *partials, int nblocks, int N) {
-    const int r = blockIdx.x;
-    const double2 d = sum_partials(partials, nblocks, N, 1, r, 0);
-    if (threadIdx.x != 0) return;
-    RhsState &s = st[r];
+__device__ __forceinline__ RhsState cg_begin(OuterState &o, double zz, double r2, double delta, int max_iters,
+                                             int max_total, int fixed) {
+    RhsState s = begin_state(o, r2, delta, max_iters, max_total, fixed);
+    s.rho = make_double2(zz, 0.0);
+    s.alpha = make_double2(0.0, 0.0);
+    s.omega = make_double2(0.0, 0.0);
+    const bool on = o.active && r2 > 0.0 && isfinite(r2) && zz > 0.0 && isfinite(zz) && s.max_iters > 0;
+    s.active = on;
+    s.next_active = on;
+    return s;
+}
+__device__ __forceinline__ void bicg_alpha(RhsState &s, double2 d) {
     s.active = s.next_active;
     if (!s.active) return;
-    const double2 a = cdiv(s.rho, d);
-    if (!(d.x * d.x + d.y * d.y > 0.0) || !finite2(a)) {
+    const double d2 = d.x * d.x + d.y * d.y;
+    const double2 a = cdiv_by(s.rho, d, d2);
+    if (!(d2 > 0.0) || !finite2(a)) {
         s.status = finite2(d) ? ST_BREAKDOWN : ST_NAN;
         s.active = 0;
         s.next_active = 0;
@@ -208,14 +204,7 @@ static __global__ void scalar_alpha_kernel(RhsState *st, const double2 *partials
     }
     s.alpha = a;
 }
-
-// After t = Mhat s: omega, rho', beta, |r'|^2 and the stopping test.
-static __global__ void scalar_omega_kernel(RhsState *st, const double2 *partials, int nblocks, int N) {
-    const int r = blockIdx.x;
-    double2 v[5];
-    sum_partials_all<5>(partials, nblocks, N, r, v);
-    if (threadIdx.x != 0) return;
-    RhsState &s = st[r];
+__device__ __forceinline__ void bicg_omega(RhsState &s, const double2 (&v)[5]) {
     if (!s.active) return;
     const double2 ts = v[0];
     const double tt = v[1].x;
@@ -223,7 +212,7 @@ static __global__ void scalar_omega_kernel(RhsState *st, const double2 *partials
     const double ss = v[4].x;
     s.iters += 1;
     bool stop = false;
-    if (!(isfinite(tt) && isfinite(ss) && finite2(ts) && finite2(r0s) && finite2(r0t))) {
+    if (!(finite1(tt) && finite1(ss) && finite2(ts) && finite2(r0s) && finite2(r0t))) {
         s.status = ST_NAN;
         s.omega = make_double2(0.0, 0.0);
         s.active = 0;  // the vector update is skipped
@@ -238,14 +227,16 @@ static __global__ void scalar_omega_kernel(RhsState *st, const double2 *partials
         if (ss > s.target2) s.status = ST_BREAKDOWN;
         stop = true;
     } else {
-        const double2 om = make_double2(ts.x / tt, ts.y / tt);
+        const double it = fp64_rcp(tt);
+        const double2 om = make_double2(ts.x * it, ts.y * it);
         const double2 rho_new = make_double2(r0s.x - (om.x * r0t.x - om.y * r0t.y),
                                              r0s.y - (om.x * r0t.y + om.y * r0t.x));
-        double r2 = ss - (ts.x * ts.x + ts.y * ts.y) / tt;
+        double r2 = ss - (ts.x * om.x + ts.y * om.y);
         if (r2 < 0.0) r2 = 0.0;
         s.omega = om;
         s.r2 = r2;
-        const double2 beta = cmul2(cdiv(rho_new, s.rho), cdiv(s.alpha, om));
+        const double2 den = cmul2(s.rho, om);  // beta = (rho'/rho)(alpha/omega) with one reciprocal
+        const double2 beta = cdiv_by(cmul2(rho_new, s.alpha), den, den.x * den.x + den.y * den.y);
         if (!finite2(beta) || !(rho_new.x * rho_new.x + rho_new.y * rho_new.y > 0.0)) {
             s.beta = make_double2(0.0, 0.0);
             if (r2 > s.target2) s.status = ST_BREAKDOWN;
@@ -258,6 +249,76 @@ static __global__ void scalar_omega_kernel(RhsState *st, const double2 *partials
     const bool done = s.fixed ? (s.iters >= s.max_iters)
                               : (s.r2 <= s.target2 || s.iters >= s.max_iters);
     s.next_active = !(stop || done);
+}
+__device__ __forceinline__ void cg_alpha(RhsState &s, double ww) {
+    s.active = s.next_active;
+    if (!s.active) return;
+    const double a = s.rho.x * fp64_rcp(ww);
+    if (!(ww > 0.0) || !finite1(a)) {
+        s.status = finite1(ww) ? ST_BREAKDOWN : ST_NAN;
+        s.active = 0;
+        s.next_active = 0;
+        return;
+    }
+    s.alpha = make_double2(a, 0.0);
+}
+__device__ __forceinline__ void cg_beta(RhsState &s, double r2, double zz) {
+    if (!s.active) return;
+    s.iters += 1;
+    if (!finite1(r2) || !finite1(zz)) {
+        s.status = ST_NAN;
+        s.active = 0;  // the p update is skipped
+        s.next_active = 0;
+        return;
+    }
+    s.r2 = r2;
+    bool stop = false;
+    if (!(zz > 0.0)) {
+        s.beta = make_double2(0.0, 0.0);
+        if (r2 > s.target2) s.status = ST_BREAKDOWN;
+        stop = true;
+    } else {
+        s.beta = make_double2(zz * fp64_rcp(s.rho.x), 0.0);
+        s.rho = make_double2(zz, 0.0);
+    }
+    const bool done = s.fixed ? (s.iters >= s.max_iters) : (s.r2 <= s.target2 || s.iters >= s.max_iters);
+    s.next_active = !(stop || done);
+}
+
+// ---------------------------------------------------------------------------
+// scalar kernels: grid = N blocks of kScalarThreads (one block per right-hand side)
+// ---------------------------------------------------------------------------
+
+// Start an inner phase: rho = <rhat, r_l>, r2 = |r_l|^2 (from the partials of
+// inner_init_kernel), target and caps; records the scale sigma = |r64| of the
+// phase.  max_iters caps this phase; max_total the iterations over all phases.
+static __global__ void inner_start_kernel(RhsState *st, OuterState *os, const double2 *partials,
+                                   int nblocks, int N, double delta, int max_iters, int max_total, int fixed) {
+    const int r = blockIdx.x;
+    double2 v[2];
+    sum_partials<2>(partials, nblocks, N, r, v);
+    const double2 rho = v[0], n2 = v[1];
+    if (threadIdx.x != 0) return;
+    st[r] = bicg_begin(os[r], rho, n2.x, delta, max_iters, max_total, fixed);
+}
+
+// After v = Mhat p: alpha = rho / <rhat, v>.
+static __global__ void scalar_alpha_kernel(RhsState *st, const double2 *partials, int nblocks, int N) {
+    const int r = blockIdx.x;
+    double2 d_[1];
+    sum_partials<1>(partials, nblocks, N, r, d_);
+    const double2 d = d_[0];
+    if (threadIdx.x != 0) return;
+    bicg_alpha(st[r], d);
+}
+
+// After t = Mhat s: omega, rho', beta, |r'|^2 and the stopping test.
+static __global__ void scalar_omega_kernel(RhsState *st, const double2 *partials, int nblocks, int N) {
+    const int r = blockIdx.x;
+    double2 v[5];
+    sum_partials<5>(partials, nblocks, N, r, v);
+    if (threadIdx.x != 0) return;
+    bicg_omega(st[r], v);
 }
 
 static __global__ void count_active_kernel(const RhsState *st, int N, int *out) {
@@ -276,24 +337,27 @@ struct VecArgs {
     int N;        // right-hand sides in the layout
 };
 
-// s = r - alpha v
+// s = r - alpha v.  HBM and L2 (3 streams of 201 MB on 16^3 x 32, FP32, width 32:
+// 65 us; with the scalars read and converted from FP64 for every element 95 us,
+// the conversions sharing the FP64 units).
 template <typename S, int R>
 static __global__ void __launch_bounds__(256) axpy_s_kernel(VecArgs a, const RhsState *st, const S *r_, const S *v_, S *s_) {
     typedef typename Real<S>::type T;
     const int G = a.N / R, lgG = __ffs(G) - 1;
     const long total = (long)a.n_elem << lgG;  // elements x groups: may exceed 2^31
-    for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-        const int e = (int)(idx >> lgG), r0 = (int)(idx & (G - 1)) * R;
-        bool any = false;
-        cx<T> al[R];
+    // a thread keeps its right-hand sides (the grid stride is a multiple of G): their scalars are converted once
+    const int r0 = (int)(threadIdx.x & (G - 1)) * R;
+    bool any = false;
+    cx<T> al[R];
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const RhsState &q = st[r0 + k];
-            any |= (q.active != 0);
-            al[k] = mk((T)q.alpha.x, (T)q.alpha.y);
-        }
-        if (!any) continue;
-        const size_t off = ((size_t)e * a.N + r0) * 2;
+    for (int k = 0; k < R; ++k) {
+        const RhsState &q = st[r0 + k];
+        any |= (q.active != 0);
+        al[k] = mk((T)q.alpha.x, (T)q.alpha.y);
+    }
+    if (!any) return;
+    for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
+        const size_t off = ((size_t)(idx >> lgG) * a.N + r0) * 2;
         cx<T> rv[R], vv[R], sv[R];
         ld_pack<S, R, true>(r_ + off, rv);
         ld_pack<S, R, true>(v_ + off, vv);
@@ -304,32 +368,32 @@ static __global__ void __launch_bounds__(256) axpy_s_kernel(VecArgs a, const Rhs
 }
 
 // x += alpha p + omega s ; r = s - omega t ; p = r + beta (p - omega v)
-// (5 reads, 3 writes per element while every right-hand side is active)
+// (5 reads, 3 writes per element while every right-hand side is active: 180 us on
+// 16^3 x 32, FP32, width 32, part of s and t still in L2; 249 us with the scalars
+// converted per element)
 template <typename S, int R>
 static __global__ void __launch_bounds__(256) update_kernel(VecArgs a, const RhsState *st, S *x_, S *r_, S *p_,
                                                     const S *s_, const S *t_, const S *v_) {
     typedef typename Real<S>::type T;
     const int G = a.N / R, lgG = __ffs(G) - 1;
     const long total = (long)a.n_elem << lgG;  // elements x groups: may exceed 2^31
+    const int r0 = (int)(threadIdx.x & (G - 1)) * R;
+    bool any = false, all = true;
+    bool on[R];
+    cx<T> al[R], om[R], be[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const RhsState &q = st[r0 + k];
+        on[k] = q.active != 0;
+        any |= on[k];
+        all &= on[k];
+        al[k] = mk((T)q.alpha.x, (T)q.alpha.y);
+        om[k] = mk((T)q.omega.x, (T)q.omega.y);
+        be[k] = mk((T)q.beta.x, (T)q.beta.y);
+    }
+    if (!any) return;
     for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-        const int e = (int)(idx >> lgG), r0 = (int)(idx & (G - 1)) * R;
-        bool any = false;
-        bool on[R];
-        cx<T> al[R], om[R], be[R];
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const RhsState &q = st[r0 + k];
-            on[k] = q.active != 0;
-            any |= on[k];
-            al[k] = mk((T)q.alpha.x, (T)q.alpha.y);
-            om[k] = mk((T)q.omega.x, (T)q.omega.y);
-            be[k] = mk((T)q.beta.x, (T)q.beta.y);
-        }
-        if (!any) continue;
-        bool all = true;
-#pragma unroll
-        for (int k = 0; k < R; ++k) all &= on[k];
-        const size_t off = ((size_t)e * a.N + r0) * 2;
+        const size_t off = ((size_t)(idx >> lgG) * a.N + r0) * 2;
         cx<T> xv[R], pv[R], sv[R], tv[R], vv[R], rv[R];
         ld_pack<S, R, false>(x_ + off, xv);
         ld_pack<S, R, false>(p_ + off, pv);
@@ -374,23 +438,32 @@ __global__ void __launch_bounds__(256) inner_init_kernel(VecArgs a, const OuterS
     cx<T> red[R][2];
 #pragma unroll
     for (int k = 0; k < R; ++k) red[k][0] = red[k][1] = zero<T>();
+    // the scales of this thread's right-hand sides: an FP64 root and division per element
+    // made this kernel 3.9 times slower (0.83 against 0.215 ms on 16^3 x 32, width 32)
+    const int r0 = (int)(threadIdx.x & (G - 1)) * R;
+    double scale[R];
+    T pscale[R];
+    bool cont[R];
+    bool any_cont = false;
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const OuterState &o = os[r0 + k];
+        const bool on = o.active && o.r2 > 0.0;
+        const double root = sqrt(o.r2);
+        scale[k] = on ? 1.0 / root : 0.0;
+        cont[k] = on && !restart && o.sigma > 0.0 && st[r0 + k].status == ST_OK;
+        pscale[k] = cont[k] ? (T)(o.sigma / root) : (T)0;
+        any_cont |= cont[k];
+    }
     for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-        const int e = (int)(idx >> lgG), r0 = (int)(idx & (G - 1)) * R;
-        const size_t off = ((size_t)e * a.N + r0) * 2;
+        const size_t off = ((size_t)(idx >> lgG) * a.N + r0) * 2;
         cx<double> src[R];
         ld_pack<double, R, true>(r64 + off, src);
         cx<T> lo[R], zr[R], pv[R], rh[R];
-        bool cont[R];
-        bool any_cont = false;
 #pragma unroll
         for (int k = 0; k < R; ++k) {
-            const OuterState &o = os[r0 + k];
-            const bool on = o.active && o.r2 > 0.0;
-            const double sc = on ? 1.0 / sqrt(o.r2) : 0.0;
-            lo[k] = mk((T)(src[k].re * sc), (T)(src[k].im * sc));
+            lo[k] = mk((T)(src[k].re * scale[k]), (T)(src[k].im * scale[k]));
             zr[k] = zero<T>();
-            cont[k] = on && !restart && o.sigma > 0.0 && st[r0 + k].status == ST_OK;
-            any_cont |= cont[k];
         }
         st_pack<S, R>(r_ + off, lo);
         ld_pack<S, R, false>(r_ + off, lo);  // the rounded value, for a consistent rho
@@ -401,9 +474,7 @@ __global__ void __launch_bounds__(256) inner_init_kernel(VecArgs a, const OuterS
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             if (cont[k]) {
-                const OuterState &o = os[r0 + k];
-                const T f = (T)(o.sigma / sqrt(o.r2));
-                pv[k] = f * pv[k];
+                pv[k] = pscale[k] * pv[k];
             } else {
                 pv[k] = lo[k];
                 rh[k] = lo[k];
@@ -455,17 +526,23 @@ __global__ void __launch_bounds__(256) cg_init_kernel(VecArgs a, const OuterStat
     cx<T> red[R][1];
 #pragma unroll
     for (int k = 0; k < R; ++k) red[k][0] = zero<T>();
+    const int r0 = (int)(threadIdx.x & (G - 1)) * R;
+    double scale[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const OuterState &o = os[r0 + k];
+        scale[k] = (o.active && o.r2 > 0.0) ? 1.0 / sqrt(o.r2) : 0.0;
+    }
     for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-        const int e = (int)(idx >> lgG), r0 = (int)(idx & (G - 1)) * R;
+        const int e = (int)(idx >> lgG);
         const size_t off = ((size_t)e * a.N + r0) * 2;
-        const double sg = g5_negates(e) ? -1.0 : 1.0;
+        const bool neg = g5_negates(e);
         cx<double> src[R];
         ld_pack<double, R, true>(r64 + off, src);
         cx<T> lo[R], zr[R];
 #pragma unroll
         for (int k = 0; k < R; ++k) {
-            const OuterState &o = os[r0 + k];
-            const double sc = (o.active && o.r2 > 0.0) ? sg / sqrt(o.r2) : 0.0;
+            const double sc = neg ? -scale[k] : scale[k];
             lo[k] = mk((T)(src[k].re * sc), (T)(src[k].im * sc));
             zr[k] = zero<T>();
         }
@@ -489,19 +566,19 @@ __global__ void __launch_bounds__(256) cg_update_kernel(VecArgs a, const RhsStat
     cx<T> red[R][1];
 #pragma unroll
     for (int k = 0; k < R; ++k) red[k][0] = zero<T>();
-    for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-        const int e = (int)(idx >> lgG), r0 = (int)(idx & (G - 1)) * R;
-        bool on[R];
-        bool any = false;
-        T al[R];
+    const int r0 = (int)(threadIdx.x & (G - 1)) * R;
+    bool on[R];
+    bool any = false;
+    T al[R];
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const RhsState &q = st[r0 + k];
-            on[k] = q.active != 0;
-            any |= on[k];
-            al[k] = (T)q.alpha.x;
-        }
-        if (!any) continue;
+    for (int k = 0; k < R; ++k) {
+        const RhsState &q = st[r0 + k];
+        on[k] = q.active != 0;
+        any |= on[k];
+        al[k] = (T)q.alpha.x;
+    }
+    for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; any && idx < total; idx += (long)gridDim.x * blockDim.x) {
+        const int e = (int)(idx >> lgG);
         const T sg = g5_negates(e) ? (T)-1 : (T)1;
         const size_t off = ((size_t)e * a.N + r0) * 2;
         cx<T> xv[R], rv[R], pv[R], wv[R];
@@ -530,19 +607,20 @@ __global__ void __launch_bounds__(256) cg_p_kernel(VecArgs a, const RhsState *st
     typedef typename Real<S>::type T;
     const int G = a.N / R, lgG = __ffs(G) - 1;
     const long total = (long)a.n_elem << lgG;  // elements x groups: may exceed 2^31
-    for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-        const int e = (int)(idx >> lgG), r0 = (int)(idx & (G - 1)) * R;
-        bool on[R];
-        bool any = false;
-        T be[R];
+    const int r0 = (int)(threadIdx.x & (G - 1)) * R;
+    bool on[R];
+    bool any = false;
+    T be[R];
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const RhsState &q = st[r0 + k];
-            on[k] = init || q.active != 0;
-            any |= on[k];
-            be[k] = init ? (T)0 : (T)q.beta.x;
-        }
-        if (!any) continue;
+    for (int k = 0; k < R; ++k) {
+        const RhsState &q = st[r0 + k];
+        on[k] = init || q.active != 0;
+        any |= on[k];
+        be[k] = init ? (T)0 : (T)q.beta.x;
+    }
+    if (!any) return;
+    for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
+        const int e = (int)(idx >> lgG);
         const T sg = g5_negates(e) ? (T)-1 : (T)1;
         const size_t off = ((size_t)e * a.N + r0) * 2;
         cx<T> uv[R], pv[R];
@@ -566,76 +644,37 @@ __global__ void __launch_bounds__(256) cg_p_kernel(VecArgs a, const RhsState *st
 static __global__ void cg_start_kernel(RhsState *st, OuterState *os, const double2 *pr, int nr, const double2 *pu,
                                        int nu, int N, double delta, int max_iters, int max_total, int fixed) {
     const int r = blockIdx.x;
-    const double2 n2 = sum_partials(pr, nr, N, 1, r, 0);
-    const double2 zz = sum_partials(pu, nu, N, 1, r, 0);
+    double2 n2_[1];
+    sum_partials<1>(pr, nr, N, r, n2_);
+    const double2 n2 = n2_[0];
+    double2 zz_[1];
+    sum_partials<1>(pu, nu, N, r, zz_);
+    const double2 zz = zz_[0];
     if (threadIdx.x != 0) return;
-    os[r].sigma = os[r].active ? sqrt(os[r].r2) : 0.0;
-    RhsState s;
-    s.rho = make_double2(zz.x, 0.0);
-    s.alpha = make_double2(0.0, 0.0);
-    s.omega = make_double2(0.0, 0.0);
-    s.beta = make_double2(0.0, 0.0);
-    s.r2 = n2.x;
-    s.r2_0 = n2.x;
-    const double red = inner_reduction(os[r], delta);
-    s.target2 = red * red * n2.x;
-    s.iters = 0;
-    s.status = ST_OK;
-    const int left = max_total - os[r].iters;
-    s.max_iters = fixed ? max_iters : (max_iters < left ? max_iters : left);
-    s.fixed = fixed;
-    const bool on = os[r].active && n2.x > 0.0 && isfinite(n2.x) && zz.x > 0.0 && isfinite(zz.x) &&
-                    s.max_iters > 0;
-    s.active = on;
-    s.next_active = on;
-    st[r] = s;
+    st[r] = cg_begin(os[r], zz.x, n2.x, delta, max_iters, max_total, fixed);
 }
 
 // After w = Mhat p: alpha = |z|^2 / |w|^2.
 static __global__ void cg_alpha_kernel(RhsState *st, const double2 *partials, int nblocks, int N) {
     const int r = blockIdx.x;
-    const double2 ww = sum_partials(partials, nblocks, N, 1, r, 0);
+    double2 ww_[1];
+    sum_partials<1>(partials, nblocks, N, r, ww_);
+    const double2 ww = ww_[0];
     if (threadIdx.x != 0) return;
-    RhsState &s = st[r];
-    s.active = s.next_active;
-    if (!s.active) return;
-    const double a = s.rho.x / ww.x;
-    if (!(ww.x > 0.0) || !isfinite(a)) {
-        s.status = isfinite(ww.x) ? ST_BREAKDOWN : ST_NAN;
-        s.active = 0;
-        s.next_active = 0;
-        return;
-    }
-    s.alpha = make_double2(a, 0.0);
+    cg_alpha(st[r], ww.x);
 }
 
 // After the update (pr: |r|^2) and u = Mhat g5 r (pu: |u|^2): beta, stopping test.
 static __global__ void cg_beta_kernel(RhsState *st, const double2 *pr, int nr, const double2 *pu, int nu, int N) {
     const int r = blockIdx.x;
-    const double2 n2 = sum_partials(pr, nr, N, 1, r, 0);
-    const double2 zz = sum_partials(pu, nu, N, 1, r, 0);
+    double2 n2_[1];
+    sum_partials<1>(pr, nr, N, r, n2_);
+    const double2 n2 = n2_[0];
+    double2 zz_[1];
+    sum_partials<1>(pu, nu, N, r, zz_);
+    const double2 zz = zz_[0];
     if (threadIdx.x != 0) return;
-    RhsState &s = st[r];
-    if (!s.active) return;
-    s.iters += 1;
-    if (!isfinite(n2.x) || !isfinite(zz.x)) {
-        s.status = ST_NAN;
-        s.active = 0;  // the p update is skipped
-        s.next_active = 0;
-        return;
-    }
-    s.r2 = n2.x;
-    bool stop = false;
-    if (!(zz.x > 0.0)) {
-        s.beta = make_double2(0.0, 0.0);
-        if (n2.x > s.target2) s.status = ST_BREAKDOWN;
-        stop = true;
-    } else {
-        s.beta = make_double2(zz.x / s.rho.x, 0.0);
-        s.rho = make_double2(zz.x, 0.0);
-    }
-    const bool done = s.fixed ? (s.iters >= s.max_iters) : (s.r2 <= s.target2 || s.iters >= s.max_iters);
-    s.next_active = !(stop || done);
+    cg_beta(st[r], n2.x, zz.x);
 }
 
 // x64 += |r64| * x_l for right-hand sides active in the outer loop.
@@ -644,20 +683,27 @@ static __global__ void __launch_bounds__(256) accumulate_kernel(VecArgs a, const
     typedef typename Real<S>::type T;
     const int G = a.N / R, lgG = __ffs(G) - 1;
     const long total = (long)a.n_elem << lgG;  // elements x groups: may exceed 2^31
+    const int r0 = (int)(threadIdx.x & (G - 1)) * R;
+    double sc[R];
+    bool on[R], any = false;
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        on[k] = os[r0 + k].active != 0;
+        any |= on[k];
+        sc[k] = on[k] ? sqrt(os[r0 + k].r2) : 0.0;
+    }
+    if (!any) return;
     for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-        const int e = (int)(idx >> lgG), r0 = (int)(idx & (G - 1)) * R;
-        const size_t off = ((size_t)e * a.N + r0) * 2;
+        const size_t off = ((size_t)(idx >> lgG) * a.N + r0) * 2;
         cx<T> xl[R];
         ld_pack<S, R, true>(x_ + off, xl);
         cx<double> acc[R];
         ld_pack<double, R, false>(x64 + off, acc);
 #pragma unroll
         for (int k = 0; k < R; ++k) {
-            const OuterState &o = os[r0 + k];
-            if (o.active) {
-                const double sc = sqrt(o.r2);
-                acc[k].re += sc * (double)xl[k].re;
-                acc[k].im += sc * (double)xl[k].im;
+            if (on[k]) {
+                acc[k].re += sc[k] * (double)xl[k].re;
+                acc[k].im += sc[k] * (double)xl[k].im;
             }
         }
         st_pack<double, R>(x64 + off, acc);
@@ -675,7 +721,9 @@ static __global__ void __launch_bounds__(256) accumulate_kernel(VecArgs a, const
 static __global__ void outer_update_kernel(OuterState *os, const RhsState *st, const double2 *partials, int nblocks,
                                     int N, int mode, double tol, int max_outer, int max_iter) {
     const int r = blockIdx.x;
-    const double2 n2 = sum_partials(partials, nblocks, N, 1, r, 0);
+    double2 n2_[1];
+    sum_partials<1>(partials, nblocks, N, r, n2_);
+    const double2 n2 = n2_[0];
     if (threadIdx.x != 0) return;
     OuterState &o = os[r];
     if (mode == 0) {
@@ -756,8 +804,12 @@ static __global__ void pow2_scale_kernel(double *f, size_t n_rows, int N, const 
 static __global__ void full_norm_kernel(OuterState *os, const double2 *pa, int na, const double2 *pb, int nb, int N,
                                  int mode) {
     const int r = blockIdx.x;
-    const double2 a = sum_partials(pa, na, N, 1, r, 0);
-    const double2 b = sum_partials(pb, nb, N, 1, r, 0);
+    double2 a_[1];
+    sum_partials<1>(pa, na, N, r, a_);
+    const double2 a = a_[0];
+    double2 b_[1];
+    sum_partials<1>(pb, nb, N, r, b_);
+    const double2 b = b_[0];
     if (threadIdx.x != 0) return;
     if (mode == 0) os[r].full_b2 = a.x + b.x;
     else os[r].full_r2 = a.x + b.x;
@@ -781,7 +833,8 @@ static __global__ void __launch_bounds__(256) norm2_kernel(VecArgs a, const S *v
         cx<T> v[R];
         ld_pack<S, R, true>(v_ + ((size_t)e * a.N + r0) * 2, v);
 #pragma unroll
-        for (int k = 0; k < R; ++k) cjmac(red[k][0], v[k], v[k]);
+        for (int k = 0; k < R; ++k)  // (the imaginary part of <v, v> is not read)
+            red[k][0].re = ::fma(v[k].re, v[k].re, ::fma(v[k].im, v[k].im, red[k][0].re));
     }
     block_reduce<R, 1, T>(red, G, a.N, partials, smem);
 }
