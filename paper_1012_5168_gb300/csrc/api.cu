@@ -149,6 +149,11 @@ struct dl_ctx {
     bool hop_tuned[5][8];
     bool autotune = true;
 };
+    bool hop_pinned[5][8];   // shapes forced by the caller: solves of that width keep to them (no resident solver)
+    // cluster-resident solver: its links per storage precision, stale after a change of the links
+    void *d_reslinks[3] = {nullptr};  // [P_F32], [P_BF16]
+    bool reslinks_ok[3] = {false, false, false};
+    int res_clusters[3][5];  // co-resident clusters of 1, 2, 4, 8, 16 blocks (-1: not asked yet)
 
 // ---------------------------------------------------------------------------
 // helpers
@@ -396,7 +401,8 @@ static int ensure_ws(dl_ctx *c, int N) {
     for (auto pp : halves)
         if (cudaMalloc((void **)pp, half) != cudaSuccess) return fail(DL_ENOMEM, "workspace allocation failed");
     for (auto &p : c->lo)
-        if (cudaMalloc(&p, half) != cudaSuccess) return fail(DL_ENOMEM, "workspace allocation failed");
+        if (cudaMalloc(&p, half + (size_t)N * 384 * 16) != cudaSuccess) return fail(DL_ENOMEM, "workspace allocation failed");
+    // (the resident solver pads each right-hand side to whole tiles of 32 sites)
     if (cudaMalloc((void **)&c->d_canon, 2 * half) != cudaSuccess) return fail(DL_ENOMEM, "workspace allocation failed");
     if (cudaMalloc((void **)&c->d_rhs, sizeof(RhsState) * N) != cudaSuccess ||
         cudaMalloc((void **)&c->d_outer, sizeof(OuterState) * N) != cudaSuccess ||
@@ -563,6 +569,7 @@ extern "C" int dl_tune_hop(dl_ctx *c, int precision, int n_rhs, int force_R, int
     const int l = ilog2(N);
     if (R_out) *R_out = c->hop_R[ip][l][2];
     if (block_out) *block_out = c->hop_block[ip][l][2];
+    c->hop_pinned[ip][l] = force_R > 0 || force_block > 0 || force_pf >= 0;
     if (pf_out) *pf_out = c->hop_kind[ip][l][2];
     if (ms_out) {
         float ms = 0.f;
@@ -600,7 +607,7 @@ extern "C" int dl_set_hop_shape(dl_ctx *c, int precision, int n_rhs, int cls, in
     c->hop_R[ip][l][m] = R;
     c->hop_block[ip][l][m] = block;
     c->hop_kind[ip][l][m] = kind;
-    c->hop_tuned[ip][l] = true;
+    c->hop_tuned[ip][l] = c->hop_pinned[ip][l] = true;
     invalidate_graphs(c);
     return DL_OK;
 }
@@ -720,10 +727,12 @@ extern "C" int dl_create(dl_ctx **out, const int dims[4], int t_bc, void *cuda_s
                 c->hop_block[p][l][m] = 128;
                 c->hop_kind[p][l][m] = 0;
             }
-            c->hop_tuned[p][l] = false;
+            c->hop_tuned[p][l] = c->hop_pinned[p][l] = false;
         }
     // coordinates table
     std::vector<uint32_t> coords(V);
+    for (auto &row : c->res_clusters)
+        for (int &v : row) v = -1;
     for (int t = 0; t < dims[3]; ++t)
         for (int z = 0; z < dims[2]; ++z)
             for (int y = 0; y < dims[1]; ++y)
@@ -778,6 +787,7 @@ extern "C" int dl_destroy(dl_ctx *c) {
                     c->d_tcol,     c->d_acc2,    c->d_clov64,   c->d_clovinv64, c->d_clovinv32, c->d_clovinv16};
     for (void *p : ptrs)
         if (p) cudaFree(p);
+                    c->d_reslinks[0], c->d_reslinks[1], c->d_reslinks[2],
     for (dl_ctx::Scratch *sc : {&c->s_phase, &c->s_site, &c->s_msum, &c->s_mloops, &c->s_mgroup, &c->s_mom,
                                 &c->s_cover, &c->s_out})
         if (sc->p) cudaFree(sc->p);
@@ -846,6 +856,7 @@ extern "C" int dl_load_gauge(dl_ctx *c, const double *U, int check) {
     return rc;
 }
 
+    for (bool &ok : c->reslinks_ok) ok = false;
 extern "C" int dl_set_kappa(dl_ctx *c, double kappa) {
     if (!c) return fail(DL_EINVAL, "null context");
     if (!std::isfinite(kappa)) return fail(DL_EINVAL, "kappa must be finite");
@@ -1241,6 +1252,61 @@ static int outer_residual(dl_ctx *c, int op, int N, const double *be, const doub
 // Solve the batch held in c->b64 (n right-hand sides, layout width N); the
 // solution is left in c->x64.  host_os receives the N outer states.
 static int solve_batch(dl_ctx *c, int n, int N, const SolveCfg &P, std::vector<OuterState> &host_os) {
+// Whether the inner phases of a solve of width N run in the cluster-resident kernel
+// (resident.cuh), with clusters of *C_out blocks.  It depends on the width alone, so
+// a ragged batch maps its right-hand sides as a full one does.  C: the smallest
+// cluster that gives every SM at most one round of sites, or the largest of which
+// N are resident at once (more clusters than fit run in waves).
+// The line.  An iteration of the resident kernel takes about 8 + 11 us per round
+// of 128 sites per SM, one of the step-by-step iteration 36 us (its eight
+// launches) + 0.5 us per 1000 (site, right-hand side) pairs.  Measured (GB300,
+// FP32 unless said, resident against step by step, a solve): 4^4, 64 right-hand
+// sides 0.72 / 1.39 ms; 4^2 x 6 x 8, 12: 1.40 / 3.18; 6 x 10 x 4 x 12 BF16, 5:
+// 2.9 / 5.4; 6^3 x 8, 32: 2.1 / 3.5; 8^3 x 16: 1: 2.5 / 3.6, 8: 4.1 / 5.1, 32: 8.6 /
+// 9.1; beyond the line 8^3 x 16, 16: 7.2 / 5.9; 12^3 x 16, 4: 7.2 / 7.3, 1: 6.3 /
+// 4.8; 12^3 x 24, 2: 10.8 / 7.9.  FP64 is bound by the FP64 units (30 / 16 ms on
+// 8^3 x 16) and the clover term's site matrices do not suit the layout (3.3 / 2.5):
+// both stay step by step, as do timed hops, pinned launch shapes, continued cycles
+// and the paired layout.
+static bool resident_plan(dl_ctx *c, const SolveCfg &P, int N, int *C_out) {
+    const int prec = P.prec;
+    if (prec == P_F64 || c->csw != 0.0 || !P.restart || c->timing || c->hop_pinned[prec][ilog2(N)] ||
+        inner_prec(c, prec, N) != prec)
+        return false;
+    int C = 0;
+    for (int l = 0; l < 5 && (C == 0 || c->Vh > (long)RES_ROUND * C); ++l) {
+        int &fit = c->res_clusters[prec][l];
+        if (fit < 0) fit = prec == P_F32 ? resident_clusters_f32(1 << l) : resident_clusters_bf16(1 << l);
+        if (fit < N) break;
+        C = 1 << l;
+    }
+    if (C == 0) return false;
+    const long rounds = (c->Vh + (long)RES_ROUND * C - 1) / ((long)RES_ROUND * C);
+    if (rounds * 23000 > 3 * 23000 + c->Vh * N || rounds > 8) return false;
+    *C_out = C;
+    return true;
+}
+
+// Tune the hops of a solve's step-by-step iterations (resident solves launch none).
+static int tune_for(dl_ctx *c, const SolveCfg &P, int N) {
+    int C = 0;
+    if (resident_plan(c, P, N, &C)) return DL_OK;
+    TRY(maybe_tune(c, P.prec, N));
+    return maybe_tune(c, P_F64, N);
+}
+
+static int ensure_resident(dl_ctx *c, int prec) {
+    if (c->reslinks_ok[prec]) return DL_OK;
+    if (!c->d_reslinks[prec] &&
+        cudaMalloc(&c->d_reslinks[prec], res_link_elems(c->Vh) * 2 * storage_bytes(prec)) != cudaSuccess)
+        return fail(DL_ENOMEM, "link allocation failed");
+    const int grid = (int)std::max<long>(1, std::min<long>((72 * c->Vh + 255) / 256, (long)c->num_sms * 8));
+    CK(launch_resident_links(prec, c->d_gauge64, c->d_coords, c->g, c->d_reslinks[prec], grid, c->cur));
+    c->kernel_launches++;
+    c->reslinks_ok[prec] = true;
+    return DL_OK;
+}
+
     const double k = c->kappa, k2 = k * k;
     // Defect-correction hops (bhat, residuals, reconstruction) in float-float
     // arithmetic for mixed-precision solves whose tolerance lies well above its
@@ -1294,10 +1360,33 @@ static int solve_batch(dl_ctx *c, int n, int N, const SolveCfg &P, std::vector<O
     for (int cycle = 0; cycle < P.max_outer; ++cycle) {
         outer_count_kernel<<<1, 1, 0, c->stream>>>(c->d_outer, N, c->d_count);
         c->kernel_launches++;
+    int res_c = 0;
+    const bool resident = resident_plan(c, P, N, &res_c);
+    if (resident) TRY(ensure_resident(c, prec));
         TRY(sync(c));
         if (*(volatile int *)c->h_count == 0) break;
         const int target = P.fixed_iters > 0 ? P.fixed_iters : P.max_iter;
-        if (P.method == DL_METHOD_CGNR) {
+        if (resident) {
+            ResArgs a;
+            for (int k = 0; k < 8; ++k) a.f[k] = c->lo[k];
+            a.links = c->d_reslinks[prec];
+            a.coords = c->d_coords;
+            a.g = c->g;
+            a.N = N;
+            a.k2 = k2;
+            a.st = c->d_rhs;
+            a.os = c->d_outer;
+            a.src = c->r64;
+            a.x64 = xe;
+            a.delta = P.delta;
+            a.max_iters = target;
+            a.max_total = P.max_iter;
+            a.fixed = P.fixed_iters > 0 ? 1 : 0;
+            const int cg = P.method == DL_METHOD_CGNR ? 1 : 0;
+            CK(prec == P_F32 ? launch_resident_f32(a, res_c, N, cg, c->stream)
+                             : launch_resident_bf16(a, res_c, N, cg, c->stream));
+            c->kernel_launches++;
+        } else if (P.method == DL_METHOD_CGNR) {
             // g5 r_l and x_l = 0; u = Mhat g5 r_l (|u|^2 = |Mhat^dag r_l|^2); p = g5 u
             VecLaunch v = vec_launch(c, prec, N, prec == P_F64 ? 16 : 8);
             CK(launch_cg_init(v, c->d_outer, c->r64, lo_ptr(c, LX), lo_ptr(c, LR), pb));
@@ -1320,7 +1409,7 @@ static int solve_batch(dl_ctx *c, int n, int N, const SolveCfg &P, std::vector<O
             c->kernel_launches += 2;
         }
         int done = 0;
-        while (done < target) {
+        while (!resident && done < target) {
             const int kk = std::min(P.chunk, target - done);
             int active = 0;
             TRY(run_chunk(c, prec, N, kk, P.use_graph, &active, P.method));
@@ -1328,8 +1417,10 @@ static int solve_batch(dl_ctx *c, int n, int N, const SolveCfg &P, std::vector<O
             if (active == 0) break;
         }
         c->cur = c->stream;
-        CK(launch_accumulate(vec_launch(c, prec, N, 0), c->d_outer, lo_ptr(c, LX), xe));
-        c->kernel_launches++;
+        if (!resident) {
+            CK(launch_accumulate(vec_launch(c, prec, N, 0), c->d_outer, lo_ptr(c, LX), xe));
+            c->kernel_launches++;
+        }
         // The true residual, every cycle, through the reconstruction of x_o.
         TRY(outer_residual(c, op, N, be, bo, xe, xo, pa, &nb));
         residual_current = true;
@@ -1356,7 +1447,6 @@ static int solve_batch(dl_ctx *c, int n, int N, const SolveCfg &P, std::vector<O
     host_os.resize(N);
     CK(cudaMemcpyAsync(host_os.data(), c->d_outer, N * sizeof(OuterState), cudaMemcpyDeviceToHost, c->stream));
     TRY(sync(c));
-    (void)n;
     return DL_OK;
 }
 
@@ -1379,8 +1469,7 @@ static int solve_impl(dl_ctx *c, const void *b, void *x, int n_rhs, const dl_sol
     const int N = std::min(P.batch, pow2_at_least(n_rhs));
     TRY(ensure_ws(c, N));
     TRY(ensure_partials(c, (size_t)2 * c->num_sms * 16 * N * 16));
-    TRY(maybe_tune(c, P.prec, N));
-    TRY(maybe_tune(c, P_F64, N));
+    TRY(tune_for(c, P, N));
     const size_t field = (size_t)c->V * 24;  // doubles per canonical field
     int worst = DL_OK;
     std::vector<OuterState> os;
@@ -2173,8 +2262,7 @@ extern "C" int dl_exact_loops(dl_ctx *c, int64_t src_first, int64_t n_src, const
     const int N = P.batch;
     TRY(ensure_ws(c, N));
     TRY(ensure_partials(c, (size_t)2 * c->num_sms * 16 * N * 16));
-    TRY(maybe_tune(c, P.prec, N));
-    TRY(maybe_tune(c, P_F64, N));
+    TRY(tune_for(c, P, N));
     c->cur = c->stream;
     // accumulators: local spin matrices [T][16] at d_acc, smeared loops [16][T] at d_acc + per
     double2 *accS = c->d_acc, *accSm = c->d_acc + per;
@@ -2382,9 +2470,8 @@ extern "C" int dl_tsm_estimate(dl_ctx *c, uint64_t seed, int n_lp, int n_hp, uns
     const int N = Plp.batch;
     TRY(ensure_ws(c, N));
     TRY(ensure_partials(c, (size_t)2 * c->num_sms * 16 * N * 16));
-    TRY(maybe_tune(c, Plp.prec, N));
-    TRY(maybe_tune(c, Php.prec, N));
-    TRY(maybe_tune(c, P_F64, N));
+    TRY(tune_for(c, Plp, N));
+    TRY(tune_for(c, Php, N));
     const size_t per_noise = (size_t)n_sinks * per;
     const size_t need = per_noise * ((size_t)n_lp + 2 * (size_t)n_hp) + 2 * per_noise;
     if (c->noise_cap < need) {
@@ -2454,8 +2541,7 @@ extern "C" int dl_dilution_error(dl_ctx *c, uint64_t seed, int n_noise, unsigned
     const int N = P.batch;
     TRY(ensure_ws(c, N));
     TRY(ensure_partials(c, (size_t)2 * c->num_sms * 16 * N * 16));
-    TRY(maybe_tune(c, P.prec, N));
-    TRY(maybe_tune(c, P_F64, N));
+    TRY(tune_for(c, P, N));
     // per-noise loops, the exact loops and the 16 results (as doubles) in the noise buffer
     const size_t need = (size_t)per * n_noise + per + 8;
     if (c->noise_cap < need) {

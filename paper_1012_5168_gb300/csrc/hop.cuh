@@ -69,17 +69,18 @@ struct HopArgs {
 };
 
 // Load the 12 components of R right-hand sides at one neighbour site and
-// project them to the two-spinor h = psi_up + s X_mu psi_down (s = SG).
-template <typename S, int R, int MU, int SG>
+// project them to the two-spinor h = psi_up + s X_mu psi_down (s = SG).  N is the
+// distance of consecutive components; NC: through the read-only path.
+template <typename S, int R, int MU, int SG, bool NC = true>
 __device__ __forceinline__ void load_project(const S *src, size_t N, cx<typename Real<S>::type> (&h)[R][6]) {
     typedef typename Real<S>::type T;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         cx<T> q0[R], q1[R], q2[R], q3[R];
-        ld_pack<S, R, true>(src + (size_t)a * N * 2, q0);
-        ld_pack<S, R, true>(src + (size_t)(3 + a) * N * 2, q1);
-        ld_pack<S, R, true>(src + (size_t)(6 + a) * N * 2, q2);
-        ld_pack<S, R, true>(src + (size_t)(9 + a) * N * 2, q3);
+        ld_pack<S, R, NC>(src + (size_t)a * N * 2, q0);
+        ld_pack<S, R, NC>(src + (size_t)(3 + a) * N * 2, q1);
+        ld_pack<S, R, NC>(src + (size_t)(6 + a) * N * 2, q2);
+        ld_pack<S, R, NC>(src + (size_t)(9 + a) * N * 2, q3);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const cx<T> p0 = q0[r], p1 = q1[r], p2 = q2[r], p3 = q3[r];

@@ -14,6 +14,7 @@
 #include "common.cuh"
 #include "hop.cuh"
 #include "blas.cuh"
+#include "resident.cuh"
 
 namespace dl {
 
@@ -141,6 +142,16 @@ cudaError_t launch_cg_update(const VecLaunch &v, const RhsState *st, void *x, vo
 cudaError_t launch_cg_p(const VecLaunch &v, const RhsState *st, const void *u, void *p, int init);
 cudaError_t launch_fill(int prec, void *x, size_t n_complex, uint32_t seed, cudaStream_t s);
 cudaError_t launch_cast(int prec, double *f64, void *lo, size_t n_complex, int to_lo, int grid, cudaStream_t s);
+// Cluster-resident solver (resident.cuh): one inner phase of n right-hand sides on
+// n clusters of C blocks (cg: CGNR, else BiCGStab), the clusters of C
+// blocks that fit the GPU at once, and the link layout it reads (36 V pairs of
+// complex values of the storage type).
+cudaError_t launch_resident_f32(const ResArgs &a, int C, int n, int cg, cudaStream_t s);
+cudaError_t launch_resident_bf16(const ResArgs &a, int C, int n, int cg, cudaStream_t s);
+int resident_clusters_f32(int C);
+int resident_clusters_bf16(int C);
+cudaError_t launch_resident_links(int prec, const double *g64, const uint32_t *coords, const Geom &g, void *out,
+                                  int grid, cudaStream_t s);
 // Clover term (clover.cu): the blocks A = 1 - kappa c_sw sum sigma F and their inverses
 // from the FP64 links (kcsw = kappa c_sw), and out = mat x in on one parity's half field
 // ([Vh][12][N] complex doubles; in place allowed), or, for acc_s != 0,
