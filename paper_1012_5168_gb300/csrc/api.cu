@@ -147,13 +147,13 @@ struct dl_ctx {
                           // packed FP32 arithmetic, 8 the same under a 128-register cap, 9 paired and
                           // warp-staged, 10 direct under a wider register cap, 11 warp-staged with two stages
     bool hop_tuned[5][8];
-    bool autotune = true;
-};
     bool hop_pinned[5][8];   // shapes forced by the caller: solves of that width keep to them (no resident solver)
     // cluster-resident solver: its links per storage precision, stale after a change of the links
     void *d_reslinks[3] = {nullptr};  // [P_F32], [P_BF16]
     bool reslinks_ok[3] = {false, false, false};
     int res_clusters[3][5];  // co-resident clusters of 1, 2, 4, 8, 16 blocks (-1: not asked yet)
+    bool autotune = true;
+};
 
 // ---------------------------------------------------------------------------
 // helpers
@@ -400,9 +400,9 @@ static int ensure_ws(dl_ctx *c, int N) {
     double **halves[] = {&c->bh64, &c->r64, &c->t64};
     for (auto pp : halves)
         if (cudaMalloc((void **)pp, half) != cudaSuccess) return fail(DL_ENOMEM, "workspace allocation failed");
+    // (the resident solver pads each right-hand side to whole tiles of 32 sites)
     for (auto &p : c->lo)
         if (cudaMalloc(&p, half + (size_t)N * 384 * 16) != cudaSuccess) return fail(DL_ENOMEM, "workspace allocation failed");
-    // (the resident solver pads each right-hand side to whole tiles of 32 sites)
     if (cudaMalloc((void **)&c->d_canon, 2 * half) != cudaSuccess) return fail(DL_ENOMEM, "workspace allocation failed");
     if (cudaMalloc((void **)&c->d_rhs, sizeof(RhsState) * N) != cudaSuccess ||
         cudaMalloc((void **)&c->d_outer, sizeof(OuterState) * N) != cudaSuccess ||
@@ -567,9 +567,9 @@ extern "C" int dl_tune_hop(dl_ctx *c, int precision, int n_rhs, int force_R, int
         return fail(DL_EINVAL, "kernel kind not available for this storage layout");
     TRY(tune_hop(c, ip, N, force_R, force_block, force_pf));
     const int l = ilog2(N);
+    c->hop_pinned[ip][l] = force_R > 0 || force_block > 0 || force_pf >= 0;
     if (R_out) *R_out = c->hop_R[ip][l][2];
     if (block_out) *block_out = c->hop_block[ip][l][2];
-    c->hop_pinned[ip][l] = force_R > 0 || force_block > 0 || force_pf >= 0;
     if (pf_out) *pf_out = c->hop_kind[ip][l][2];
     if (ms_out) {
         float ms = 0.f;
@@ -729,10 +729,10 @@ extern "C" int dl_create(dl_ctx **out, const int dims[4], int t_bc, void *cuda_s
             }
             c->hop_tuned[p][l] = c->hop_pinned[p][l] = false;
         }
-    // coordinates table
-    std::vector<uint32_t> coords(V);
     for (auto &row : c->res_clusters)
         for (int &v : row) v = -1;
+    // coordinates table
+    std::vector<uint32_t> coords(V);
     for (int t = 0; t < dims[3]; ++t)
         for (int z = 0; z < dims[2]; ++z)
             for (int y = 0; y < dims[1]; ++y)
@@ -784,10 +784,10 @@ extern "C" int dl_destroy(dl_ctx *c) {
     void *ptrs[] = {c->d_coords,   c->d_gauge64, c->d_gauge32,  c->d_gauge16, c->d_gauge8_32, c->d_gauge8_16, c->d_gauge8q,
                     c->d_gauge8d,
                     c->d_gauge_ff, c->d_gammas,  c->d_partials, c->d_acc,     c->d_noise,     c->d_w,
+                    c->d_reslinks[0], c->d_reslinks[1], c->d_reslinks[2],
                     c->d_tcol,     c->d_acc2,    c->d_clov64,   c->d_clovinv64, c->d_clovinv32, c->d_clovinv16};
     for (void *p : ptrs)
         if (p) cudaFree(p);
-                    c->d_reslinks[0], c->d_reslinks[1], c->d_reslinks[2],
     for (dl_ctx::Scratch *sc : {&c->s_phase, &c->s_site, &c->s_msum, &c->s_mloops, &c->s_mgroup, &c->s_mom,
                                 &c->s_cover, &c->s_out})
         if (sc->p) cudaFree(sc->p);
@@ -853,10 +853,10 @@ extern "C" int dl_load_gauge(dl_ctx *c, const double *U, int check) {
     cudaFree(tmp);
     if (rc == DL_OK) c->have_gauge = true;
     c->clover_stale = true;
+    for (bool &ok : c->reslinks_ok) ok = false;
     return rc;
 }
 
-    for (bool &ok : c->reslinks_ok) ok = false;
 extern "C" int dl_set_kappa(dl_ctx *c, double kappa) {
     if (!c) return fail(DL_EINVAL, "null context");
     if (!std::isfinite(kappa)) return fail(DL_EINVAL, "kappa must be finite");
@@ -1249,9 +1249,6 @@ static int outer_residual(dl_ctx *c, int op, int N, const double *be, const doub
     return do_hop(c, op, MODE_RESID, RED_NORM, c->r64, xo, xe, be, nullptr, 0, N, -k, 0, Vh, pa, nb);
 }
 
-// Solve the batch held in c->b64 (n right-hand sides, layout width N); the
-// solution is left in c->x64.  host_os receives the N outer states.
-static int solve_batch(dl_ctx *c, int n, int N, const SolveCfg &P, std::vector<OuterState> &host_os) {
 // Whether the inner phases of a solve of width N run in the cluster-resident kernel
 // (resident.cuh), with clusters of *C_out blocks.  It depends on the width alone, so
 // a ragged batch maps its right-hand sides as a full one does.  C: the smallest
@@ -1307,6 +1304,9 @@ static int ensure_resident(dl_ctx *c, int prec) {
     return DL_OK;
 }
 
+// Solve the batch held in c->b64 (n right-hand sides, layout width N); the
+// solution is left in c->x64.  host_os receives the N outer states.
+static int solve_batch(dl_ctx *c, int n, int N, const SolveCfg &P, std::vector<OuterState> &host_os) {
     const double k = c->kappa, k2 = k * k;
     // Defect-correction hops (bhat, residuals, reconstruction) in float-float
     // arithmetic for mixed-precision solves whose tolerance lies well above its
@@ -1357,12 +1357,12 @@ static int ensure_resident(dl_ctx *c, int prec) {
     CK(cudaMemsetAsync(xe, 0, half * sizeof(double), c->stream));
     bool residual_current = false;  // c->r64 and x_o belong to the current x_e
     const int prec = inner_prec(c, P.prec, N);
-    for (int cycle = 0; cycle < P.max_outer; ++cycle) {
-        outer_count_kernel<<<1, 1, 0, c->stream>>>(c->d_outer, N, c->d_count);
-        c->kernel_launches++;
     int res_c = 0;
     const bool resident = resident_plan(c, P, N, &res_c);
     if (resident) TRY(ensure_resident(c, prec));
+    for (int cycle = 0; cycle < P.max_outer; ++cycle) {
+        outer_count_kernel<<<1, 1, 0, c->stream>>>(c->d_outer, N, c->d_count);
+        c->kernel_launches++;
         TRY(sync(c));
         if (*(volatile int *)c->h_count == 0) break;
         const int target = P.fixed_iters > 0 ? P.fixed_iters : P.max_iter;
