@@ -119,7 +119,7 @@ struct dl_ctx {
     size_t noise_cap = 0;
     double2 *d_w = nullptr;      // gamma weights / spin matrices
     size_t w_cap = 0;
-    int *d_tcol = nullptr;       // per-column timeslice of the current batch (64 ints)
+    int *d_tcol = nullptr;       // per-column timeslice of the current batch (64 ints), then of its groups (64)
     // momentum projection and correlators (grown on demand)
     struct Scratch {
         void *p = nullptr;
@@ -752,7 +752,7 @@ extern "C" int dl_create(dl_ctx **out, const int dims[4], int t_bc, void *cuda_s
     if (cudaMalloc((void **)&c->d_coords, V * sizeof(uint32_t)) != cudaSuccess ||
         cudaMalloc((void **)&c->d_gammas, 256 * sizeof(double2)) != cudaSuccess ||
         cudaMalloc((void **)&c->d_acc, 2 * 16 * dims[3] * sizeof(double2)) != cudaSuccess ||
-        cudaMalloc((void **)&c->d_tcol, 64 * sizeof(int)) != cudaSuccess ||
+        cudaMalloc((void **)&c->d_tcol, 128 * sizeof(int)) != cudaSuccess ||
         cudaMalloc((void **)&c->d_acc2, (size_t)64 * 2 * 16 * dims[3] * sizeof(double2)) != cudaSuccess ||
         cudaHostAlloc((void **)&c->h_count, sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer((void **)&c->d_count, c->h_count, 0) != cudaSuccess ||
@@ -1895,18 +1895,39 @@ static int contract_eo(dl_ctx *c, const double *eta, const double *phi, int n, i
 }
 
 // Momentum-projected contraction (momentum.cuh): site spin matrices, their
-// Fourier sums against the phase table, Gamma traces into dst[j][q][16][T].
+// Fourier sums against the phase table, Gamma traces into dst[slot][q][16][T],
+// one slot per group of `group` right-hand sides.
 struct MomSpec {
-    int n_mom;
-    const double2 *phase;  // [n_mom][V3]
-    double2 *site;         // [N][nt][V3][16]
-    double2 *msum;         // [N][nt][n_mom][16]
+    int n_mom, n_rep;
+    const double2 *phase;  // [n_rep][V3]
+    const int *zero;       // [n_rep]: 1 for zero momentum
+    const int *rep;        // [n_mom]: representative << 1 | negated
+    int group;             // right-hand sides summed at the sites (1: none)
+    const int *tgrp;       // with time dilution: the timeslice of each slot
+    double2 *site;         // [slots][nt][16][V3]
+    FourierSum *msum;         // [slots][nt][16][n_rep]
     double2 *dst;          // [sink slot][N][n_mom][16][T]
 };
 
+// Fourier sums and traces of `slots` site matrices held in m.site.
+static int mom_finish(dl_ctx *c, int slots, int nt, int t_lo, const MomSpec &m, double2 *dst) {
+    const int T = c->dims[3];
+    const int V3 = c->dims[0] * c->dims[1] * c->dims[2];
+    const long rows = (long)slots * nt * 16;
+    fourier_kernel<1><<<dim3((unsigned)((rows + 3) / 4), (m.n_rep + 3) / 4), 128, 0, c->cur>>>(
+        m.site, m.phase, m.zero, V3, rows, m.n_rep, m.msum);
+    const int cnt = slots * m.n_mom * 16 * T;
+    zero_kernel<<<std::max(1, (cnt + 255) / 256), 256, 0, c->cur>>>(dst, cnt);
+    const int tot = slots * nt * m.n_mom * 16;
+    mom_gamma_kernel<<<std::max(1, (tot + 255) / 256), 256, 0, c->cur>>>(m.msum, c->d_gammas, m.rep, m.n_rep, slots, nt,
+                                                                         m.n_mom, T, t_lo, m.tgrp, dst);
+    c->kernel_launches += 3;
+    CK(cudaGetLastError());
+    return DL_OK;
+}
+
 static int contract_mom_eo(dl_ctx *c, const double *eta, const double *phi, int n, int N, int t_lo, int t_hi,
                            const MomSpec &m, double2 *dst, const int *tcol) {
-    const int T = c->dims[3];
     const int V3 = c->dims[0] * c->dims[1] * c->dims[2];
     const int nt = tcol ? 1 : t_hi - t_lo;
     SiteSpinArgs A;
@@ -1922,16 +1943,31 @@ static int contract_mom_eo(dl_ctx *c, const double *eta, const double *phi, int 
     A.out = m.site;
     Launch l = make_launch(c, (long)nt * 2 * c->g.V3h * n, 128, 0, 8);
     site_spin_kernel<<<l.grid, l.block, 0, c->cur>>>(A);
-    fourier_kernel<<<dim3(n * nt, (m.n_mom * 16 + 255) / 256), 256, 0, c->cur>>>(m.site, m.phase, V3, 16, m.n_mom,
-                                                                                 m.msum);
-    const int cnt = n * m.n_mom * 16 * T;
-    zero_kernel<<<std::max(1, (cnt + 255) / 256), 256, 0, c->cur>>>(dst, cnt);
-    const int tot = n * nt * m.n_mom * 16;
-    mom_gamma_kernel<<<std::max(1, (tot + 255) / 256), 256, 0, c->cur>>>(m.msum, c->d_gammas, n, nt, m.n_mom, T,
-                                                                         A.t_lo, tcol, dst);
-    c->kernel_launches += 4;
-    CK(cudaGetLastError());
-    return DL_OK;
+    c->kernel_launches++;
+    if (m.group > 1) {
+        const long per = (long)nt * 16 * V3;
+        group_site_kernel<<<(int)std::min<long>((per + 255) / 256, (long)c->num_sms * 8), 256, 0, c->cur>>>(
+            m.site, per, n / m.group, m.group);
+        c->kernel_launches++;
+    }
+    return mom_finish(c, n / m.group, nt, A.t_lo, m, dst);
+}
+
+// The local sink from canonical fields (no conversion).
+static int contract_mom_canon(dl_ctx *c, const double *eta, const double *phi, int n, const MomSpec &m, double2 *dst) {
+    const int V3 = c->dims[0] * c->dims[1] * c->dims[2];
+    CanonSpinArgs A;
+    A.eta = reinterpret_cast<const double2 *>(eta);
+    A.phi = reinterpret_cast<const double2 *>(phi);
+    A.g = c->g;
+    A.V3 = V3;
+    A.group = m.group;
+    A.nt = m.tgrp ? 1 : c->dims[3];
+    A.tgrp = m.tgrp;
+    A.out = m.site;
+    canon_spin_kernel<<<dim3((V3 + 31) / 32, A.nt, n / m.group), 256, 0, c->cur>>>(A);
+    c->kernel_launches++;
+    return mom_finish(c, n / m.group, A.nt, 0, m, dst);
 }
 
 // Loops of the EO pair (eta in *eta_buf, phi in *phi_buf) for the requested
@@ -2102,16 +2138,54 @@ static int ensure_scratch(dl_ctx::Scratch &sc, size_t bytes) {
 }
 
 // Upload n_mom momenta and build the phase table exp(-i p.(x - o)) on the device.
-static int build_phases(dl_ctx *c, const int *momenta, int n_mom, int ox, int oy, int oz) {
+// Momenta that differ by a sign share a representative (their phases are complex
+// conjugates): *n_rep_out of them.  c->s_mom holds the representatives' integers
+// [n_rep][3], their zero flags [n_rep] and, per momentum, representative << 1 | negated.
+static int build_phases(dl_ctx *c, const int *momenta, int n_mom, int ox, int oy, int oz, MomSpec *m) {
     const int V3 = c->dims[0] * c->dims[1] * c->dims[2];
-    TRY(ensure_scratch(c->s_mom, sizeof(int) * 3 * n_mom));
-    TRY(ensure_scratch(c->s_phase, sizeof(double2) * (size_t)n_mom * V3));
-    CK(cudaMemcpyAsync(c->s_mom.p, momenta, sizeof(int) * 3 * n_mom, cudaMemcpyHostToDevice, c->stream));
-    const int tot = n_mom * V3;
+    std::vector<int> reps, zero, map(n_mom);
+    auto wrap = [&](int v, int mu) { return ((v % c->dims[mu]) + c->dims[mu]) % c->dims[mu]; };
+    for (int q = 0; q < n_mom; ++q) {
+        const int *p = momenta + 3 * q;
+        int found = -1;
+        for (size_t r = 0; r < zero.size() && found < 0; ++r) {
+            bool same = true, neg = true;
+            for (int mu = 0; mu < 3; ++mu) {
+                same &= wrap(p[mu], mu) == wrap(reps[3 * r + mu], mu);
+                neg &= wrap(-(p[mu] % c->dims[mu]), mu) == wrap(reps[3 * r + mu], mu);
+            }
+            if (same || neg) found = (int)r * 2 + (same ? 0 : 1);
+        }
+        if (found < 0) {
+            found = (int)zero.size() * 2;
+            bool z = true;
+            for (int mu = 0; mu < 3; ++mu) {
+                reps.push_back(p[mu]);
+                z &= wrap(p[mu], mu) == 0;
+            }
+            zero.push_back(z ? 1 : 0);
+        }
+        map[q] = found;
+    }
+    const int nr = (int)zero.size();
+    std::vector<int> all(reps);
+    all.insert(all.end(), zero.begin(), zero.end());
+    all.insert(all.end(), map.begin(), map.end());
+    TRY(ensure_scratch(c->s_mom, sizeof(int) * all.size()));
+    TRY(ensure_scratch(c->s_phase, sizeof(double2) * (size_t)nr * V3));
+    CK(cudaMemcpyAsync(c->s_mom.p, all.data(), sizeof(int) * all.size(), cudaMemcpyHostToDevice, c->stream));
+    const int tot = nr * V3;
     phase_table_kernel<<<std::max(1, std::min((tot + 255) / 256, 8 * c->num_sms)), 256, 0, c->stream>>>(
-        (double2 *)c->s_phase.p, (const int *)c->s_mom.p, n_mom, c->g, ox, oy, oz);
+        (double2 *)c->s_phase.p, (const int *)c->s_mom.p, nr, c->g, ox, oy, oz);
     c->kernel_launches++;
     CK(cudaGetLastError());
+    m->n_mom = n_mom;
+    m->n_rep = nr;
+    m->phase = (const double2 *)c->s_phase.p;
+    m->zero = (const int *)c->s_mom.p + 3 * nr;
+    m->rep = m->zero + nr;
+    m->group = 1;
+    m->tgrp = nullptr;
     return DL_OK;
 }
 
@@ -2139,35 +2213,50 @@ extern "C" int dl_trace_loops_mom(dl_ctx *c, const void *eta, const void *phi, i
     const int N = std::min(64, pow2_at_least(n_rhs));
     const int per_batch = (N / group) * group;
     const int nt = t_of_rhs ? 1 : T;
-    TRY(ensure_ws(c, N));
-    TRY(build_phases(c, momenta, n_mom, 0, 0, 0));
-    TRY(ensure_scratch(c->s_site, sizeof(double2) * (size_t)N * nt * V3 * 16));
-    TRY(ensure_scratch(c->s_msum, sizeof(double2) * (size_t)N * nt * n_mom * 16));
+    const bool local = (sink & DL_SINK_LOCAL) != 0, smeared = (sink & DL_SINK_SMEARED) != 0;
+    // A group whose pairs share their timeslices is summed at the sites, before the Fourier sums.
+    bool at_sites = true;
+    if (t_of_rhs)
+        for (int j = 0; j < n_rhs; ++j) at_sites &= t_of_rhs[j] == t_of_rhs[j - j % group];
+    const int sum = at_sites ? group : 1, slots = N / sum;
+    if (smeared) TRY(ensure_ws(c, N));
+    MomSpec m;
+    TRY(build_phases(c, momenta, n_mom, 0, 0, 0, &m));
+    m.group = sum;
+    TRY(ensure_scratch(c->s_site, sizeof(double2) * (size_t)(smeared ? N : slots) * nt * V3 * 16));
+    TRY(ensure_scratch(c->s_msum, sizeof(FourierSum) * (size_t)slots * nt * m.n_rep * 16));
     TRY(ensure_scratch(c->s_mloops, sizeof(double2) * (size_t)n_sinks * N * per));
     TRY(ensure_scratch(c->s_mgroup, sizeof(double2) * (size_t)N * n_sinks * per));
-    MomSpec m;
-    m.n_mom = n_mom;
-    m.phase = (const double2 *)c->s_phase.p;
     m.site = (double2 *)c->s_site.p;
-    m.msum = (double2 *)c->s_msum.p;
+    m.msum = (FourierSum *)c->s_msum.p;
     m.dst = (double2 *)c->s_mloops.p;
     const size_t field = (size_t)c->V * 24;
     const int cb0 = 0, cb1 = t_of_rhs ? c->g.V3h : (int)c->Vh;
     c->cur = c->stream;
     int g_done = 0;
+    int ts[128];  // timeslice of each right-hand side of the batch, then of each slot
     for (int j0 = 0; j0 < n_rhs; j0 += per_batch) {
         const int n = std::min(per_batch, n_rhs - j0);
         const int *tcol = nullptr;
         if (t_of_rhs) {
-            CK(cudaMemcpyAsync(c->d_tcol, t_of_rhs + j0, n * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+            for (int j = 0; j < n; ++j) ts[j] = t_of_rhs[j0 + j];
+            for (int k = 0; k < n / sum; ++k) ts[64 + k] = t_of_rhs[j0 + k * sum];
+            CK(cudaMemcpyAsync(c->d_tcol, ts, sizeof(ts), cudaMemcpyHostToDevice, c->stream));
             tcol = c->d_tcol;
+            m.tgrp = c->d_tcol + 64;
         }
-        TRY(canon_to_eo(c, (const double *)eta + j0 * field, c->b64, n, N, 0, cb0, cb1, tcol));
-        TRY(canon_to_eo(c, (const double *)phi + j0 * field, c->x64, n, N, 0, cb0, cb1, tcol));
-        TRY(trace_eo(c, c->b64, c->x64, n, N, sink, sm, 0, T, n_sinks, tcol, &m));
+        const double *e = (const double *)eta + j0 * field, *f = (const double *)phi + j0 * field;
+        if (local) TRY(contract_mom_canon(c, e, f, n, m, m.dst));
+        if (smeared) {
+            TRY(canon_to_eo(c, e, c->b64, n, N, 0, cb0, cb1, tcol));
+            TRY(canon_to_eo(c, f, c->x64, n, N, 0, cb0, cb1, tcol));
+            MomSpec ms = m;
+            ms.dst = m.dst + (local ? (size_t)N * per : 0);
+            TRY(trace_eo(c, c->b64, c->x64, n, N, DL_SINK_SMEARED, sm, 0, T, 1, tcol, &ms));
+        }
         const int ng = n / group;
         group_sum_kernel<<<std::max(1, (ng * n_sinks * per + 255) / 256), 256, 0, c->stream>>>(
-            m.dst, n, N, group, n_sinks, per, (double2 *)c->s_mgroup.p);
+            m.dst, n / sum, N, group / sum, n_sinks, per, (double2 *)c->s_mgroup.p);
         c->kernel_launches++;
         CK(cudaMemcpyAsync(host_out + (size_t)g_done * n_sinks * per * 2, c->s_mgroup.p,
                            sizeof(double2) * (size_t)ng * n_sinks * per, cudaMemcpyDeviceToHost, c->stream));
@@ -2187,18 +2276,21 @@ extern "C" int dl_meson_correlators(dl_ctx *c, const void *prop, const int src[4
     const int T = c->dims[3];
     const int V3 = c->dims[0] * c->dims[1] * c->dims[2];
     c->cur = c->stream;
-    TRY(build_phases(c, momenta, n_mom, src[0], src[1], src[2]));
-    TRY(ensure_scratch(c->s_site, sizeof(double2) * (size_t)c->V * 256));
-    TRY(ensure_scratch(c->s_msum, sizeof(double2) * (size_t)T * n_mom * 256));
+    MomSpec m;
+    TRY(build_phases(c, momenta, n_mom, src[0], src[1], src[2], &m));
+    TRY(ensure_scratch(c->s_site, sizeof(double2) * (size_t)c->V * MESON_E));
+    TRY(ensure_scratch(c->s_msum, sizeof(FourierSum) * (size_t)T * m.n_rep * MESON_E));
     TRY(ensure_scratch(c->s_out, sizeof(double2) * (size_t)n_mom * 256 * T));
-    Launch l = make_launch(c, c->V * 16, 128, 0, 8);
-    meson_site_kernel<<<l.grid, l.block, 0, c->stream>>>((const double *)prop, c->V, (double2 *)c->s_site.p);
-    fourier_kernel<<<dim3(T, n_mom), 256, 0, c->stream>>>((const double2 *)c->s_site.p,
-                                                          (const double2 *)c->s_phase.p, V3, 256, n_mom,
-                                                          (double2 *)c->s_msum.p);
+    const size_t smem = 144 * 33 * sizeof(double2);
+    CK(cudaFuncSetAttribute(meson_site_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    meson_site_kernel<<<(int)((c->V + 31) / 32), 320, smem, c->stream>>>((const double2 *)prop, (int)c->V, V3,
+                                                                        (double2 *)c->s_site.p);
+    const long rows = (long)T * MESON_E;
+    fourier_kernel<2><<<dim3((unsigned)((rows + 7) / 8), (m.n_rep + 3) / 4), 128, 0, c->stream>>>(
+        (const double2 *)c->s_site.p, m.phase, m.zero, V3, rows, m.n_rep, (FourierSum *)c->s_msum.p);
     const int tot = n_mom * 256 * T;
     meson_gamma_kernel<<<std::max(1, std::min((tot + 255) / 256, 8 * c->num_sms)), 256, 0, c->stream>>>(
-        (const double2 *)c->s_msum.p, c->d_gammas, T, n_mom, src[3], (double2 *)c->s_out.p);
+        (const FourierSum *)c->s_msum.p, c->d_gammas, m.rep, m.n_rep, T, n_mom, src[3], (double2 *)c->s_out.p);
     c->kernel_launches += 3;
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(host_out, c->s_out.p, sizeof(double2) * (size_t)tot, cudaMemcpyDeviceToHost, c->stream));

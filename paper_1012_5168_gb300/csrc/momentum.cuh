@@ -5,9 +5,9 @@
 // and the connected meson function of a point source at y (o = y):
 //     C^{BA}(p, t) = - sum_x exp(-i p.(x - y)) Tr[g5 S(x)^dag g5 Gamma_B S(x) Gamma_A].
 // Both run in three steps: a per-site matrix (the 4x4 spin matrix
-// phi eta^dag, or the 16x16 colour-summed product of the propagator with its
-// conjugate), its Fourier sum over each timeslice against a phase table, and the
-// Gamma traces.  All sums are FP64 in a fixed order.  The disconnected
+// phi eta^dag summed over a group of pairs, or the hermitian 16x16 colour-summed
+// product of the propagator with its conjugate), its Fourier sums over each
+// timeslice against a phase table, and the Gamma traces.  All sums are FP64 in a fixed order.  The disconnected
 // function combines per-noise loops at p and -p over pairs of distinct noise
 // vectors, so no noise vector is multiplied with itself.
 #pragma once
@@ -41,7 +41,7 @@ struct SiteSpinArgs {
     int N, n;           // layout width, right-hand sides in use
     int t_lo, nt;       // timeslices t_lo .. t_lo + nt - 1 (nt = 1 with tcol)
     const int *tcol;    // if set: right-hand side j lives on timeslice tcol[j]
-    double2 *out;       // [n][nt][V3][16]: S_{beta alpha}(x) = sum_a phi_{beta a}(x) conj(eta_{alpha a}(x))
+    double2 *out;       // [n][nt][16][V3]: S_{beta alpha}(x) = sum_a phi_{beta a}(x) conj(eta_{alpha a}(x))
 };
 
 // One thread per (site of the timeslice, right-hand side); j is the fastest
@@ -70,7 +70,7 @@ static __global__ void site_spin_kernel(SiteSpinArgs A) {
             ld_pack<double, 1, true>(A.phi + base + (size_t)c * A.N * 2, v);
             f[c] = v[0];
         }
-        double2 *o = A.out + (((size_t)j * A.nt + tt) * V3 + s) * 16;
+        double2 *o = A.out + ((size_t)j * A.nt + tt) * 16 * V3 + s;
 #pragma unroll
         for (int be = 0; be < 4; ++be)
 #pragma unroll
@@ -78,43 +78,215 @@ static __global__ void site_spin_kernel(SiteSpinArgs A) {
                 cx<double> acc = zero<double>();
 #pragma unroll
                 for (int a = 0; a < 3; ++a) cjmac(acc, e[3 * al + a], f[3 * be + a]);
-                o[be * 4 + al] = make_double2(acc.re, acc.im);
+                o[(size_t)(be * 4 + al) * V3] = make_double2(acc.re, acc.im);
             }
     }
 }
 
-// out[jt][q][e] = sum_s ph[q][s] in[jt][s][e]; grid = (J*nt, ceil(Q*E / blockDim.x)).
-static __global__ void fourier_kernel(const double2 *in, const double2 *ph, int V3, int E, int Q, double2 *out) {
-    const int jt = blockIdx.x;
-    const int o = blockIdx.y * blockDim.x + threadIdx.x;
-    if (o >= Q * E) return;
-    const int q = o / E, e = o % E;
-    const double2 *src = in + (size_t)jt * V3 * E + e;
-    const double2 *w = ph + (size_t)q * V3;
-    double re = 0.0, im = 0.0;
-    for (int s = 0; s < V3; ++s) {
-        const double2 a = __ldg(w + s), b = __ldg(src + (size_t)s * E);
-        re = ::fma(a.x, b.x, ::fma(-a.y, b.y, re));
-        im = ::fma(a.x, b.y, ::fma(a.y, b.x, im));
+// site[g] = sum of the site matrices of each run of `group` right-hand sides (fixed order,
+// in place: slot g lies in a group that is summed no later than g).
+static __global__ void group_site_kernel(double2 *site, long per, int ng, int group) {
+    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < per; i += (long)gridDim.x * blockDim.x)
+        for (int g = 0; g < ng; ++g) {
+            double re = 0.0, im = 0.0;
+            for (int k = 0; k < group; ++k) {
+                const double2 v = site[(size_t)(g * group + k) * per + i];
+                re += v.x;
+                im += v.y;
+            }
+            site[(size_t)g * per + i] = make_double2(re, im);
+        }
+}
+
+// Site matrices of a whole group of pairs straight from canonical fields:
+//   out[g][tt][16][V3] = sum_{j in group g} sum_a phi_{beta a}(x) conj(eta_{alpha a}(x)).
+// Everything after it is linear, so summing the group's pairs here divides the
+// Fourier sums and their input by the group size, and no field is converted.
+//
+// A block of eight warps takes 32 sites and walks the group's pairs: both fields'
+// tiles ([32][12] complex, one contiguous run each) go through shared memory, the
+// next pair's loads in flight while the current one is multiplied.  Warp w works
+// for source spin w & 3 and, of every pair of neighbouring sites, the one of parity
+// w >> 2; a lane for (site, beta), so the three products of a colour are one
+// warp-wide decision: where a diluted eta vanishes for the whole warp the FP64
+// work is left out (dense fields are bound by FP64: 192 FMA a site and pair, 1.2 ms
+// for 48 pairs on 16^3 x 32; diluted ones by reading the fields, 0.36 ms), except
+// that a non-finite phi still makes the sum NaN, as 0 times it would.
+struct CanonSpinArgs {
+    const double2 *eta, *phi;  // canonical [n][V][12]
+    Geom g;
+    int V3, group, nt;         // nt timeslices from 0, or (tgrp) one timeslice per group
+    const int *tgrp;
+    double2 *out;
+};
+__device__ __forceinline__ bool cx_nonzero(double2 z) {
+    return (((unsigned)__double2hiint(z.x) | (unsigned)__double2hiint(z.y)) << 1 | (unsigned)__double2loint(z.x) |
+            (unsigned)__double2loint(z.y)) != 0u;
+}
+__device__ __forceinline__ bool cx_bad(double2 z) {  // infinite or NaN, without FP64 instructions
+    return (__double2hiint(z.x) & 0x7ff00000) == 0x7ff00000 || (__double2hiint(z.y) & 0x7ff00000) == 0x7ff00000;
+}
+static __global__ void __launch_bounds__(256) canon_spin_kernel(CanonSpinArgs A) {
+    __shared__ double2 se[2][384], sf[2][384];
+    const int tile = blockIdx.x, tt = blockIdx.y, gi = blockIdx.z;
+    const int t = A.tgrp ? A.tgrp[gi] : tt;
+    const int s0 = tile * 32, ns = min(32, A.V3 - s0);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, al = w & 3, par = w >> 2, be = lane & 3;
+    const long V = (long)A.V3 * A.g.L[3];
+    const size_t first = ((size_t)gi * A.group * V + (size_t)t * A.V3 + s0) * 12;
+    // the two sites of this lane: of the pairs lane / 4 and lane / 4 + 8, the one of parity par
+    int site[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int m = (lane >> 2) + 8 * h, i0 = t * A.V3 + s0 + 2 * m;
+        const int y = i0 / A.g.L[0], z = y / A.g.L[1], u = z / A.g.L[2];  // (x of an even site is even)
+        site[h] = 2 * m + ((par + y + z + u) & 1);
     }
-    out[((size_t)jt * Q + q) * E + e] = make_double2(re, im);
+    cx<double> acc[2] = {zero<double>(), zero<double>()};
+    bool bad = false;
+    const int ne = ns * 12;  // 384 elements a tile: thread k loads elements k and k + 256 of both fields
+    double2 r[4];
+    auto load = [&](int j) {
+        const size_t o = first + (size_t)j * V * 12;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = threadIdx.x + 256 * h;
+            if (k < ne) {
+                r[2 * h] = __ldg(A.eta + o + k);
+                r[2 * h + 1] = __ldg(A.phi + o + k);
+            }
+        }
+    };
+    load(0);
+    for (int j = 0; j < A.group; ++j) {
+        const int b = j & 1;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = threadIdx.x + 256 * h;
+            if (k < ne) {
+                se[b][k] = r[2 * h];
+                sf[b][k] = r[2 * h + 1];
+            }
+        }
+        __syncthreads();  // (buffer b was last read two steps ago, before the previous barrier)
+        if (j + 1 < A.group) load(j + 1);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const bool in = site[h] < ns;
+            const int o = (in ? site[h] : 0) * 12;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const double2 e = se[b][o + 3 * al + a], f = sf[b][o + 3 * be + a];
+                if (__any_sync(0xffffffffu, in && cx_nonzero(e)))
+                    cjmac(acc[h], mk(e.x, e.y), mk(f.x, f.y));
+                else
+                    bad |= in && cx_bad(f);
+            }
+        }
+    }
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    double2 *o = A.out + (((size_t)gi * A.nt + tt) * 16 + be * 4 + al) * A.V3 + s0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (site[h] < ns) o[site[h]] = bad ? make_double2(nan, nan) : make_double2(acc[h].re, acc[h].im);
+}
+
+struct __align__(16) FourierSum {
+    double x, y, z, w;  // sums of c x, s y, c y, s x
+};
+
+// Fourier sums over a timeslice.  Momenta come as representatives r with
+// phases e^{-i p.x} = c + i s; p and -p share one (conjugate phases), and the four
+// real sums
+//   out[row][r] = (sum c x, sum s y, sum c y, sum s x)   of  z = x + i y = in[row][site]
+// give the sums of z and of conj(z) at p and at -p.  in: [rows][V3] (a row is one
+// matrix entry on one timeslice).  A warp takes EPW rows and up to four
+// representatives (blockIdx.y picks which): its lanes walk the sites (coalesced,
+// each phase used for EPW rows), and the lane sums meet in a fixed order.  A
+// representative with zero momentum (zero[r]) needs sums of x and y only.
+template <int EPW>
+static __global__ void __launch_bounds__(128) fourier_kernel(const double2 *in, const double2 *ph, const int *zero,
+                                                             int V3, long rows, int n_rep, FourierSum *out) {
+    const int lane = threadIdx.x & 31;
+    const long row = ((long)blockIdx.x * 4 + (threadIdx.x >> 5)) * EPW;
+    const int r0 = blockIdx.y * 4;
+    if (row >= rows) return;
+    FourierSum acc[EPW][4];
+    bool z[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        z[r] = r0 + r < n_rep && zero[r0 + r] != 0;
+#pragma unroll
+        for (int e = 0; e < EPW; ++e) acc[e][r] = FourierSum{0.0, 0.0, 0.0, 0.0};
+    }
+    for (int s = lane; s < V3; s += 32) {
+        double2 v[EPW];
+#pragma unroll
+        for (int e = 0; e < EPW; ++e) v[e] = row + e < rows ? __ldg(in + (size_t)(row + e) * V3 + s) : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            if (r0 + r >= n_rep) break;
+            if (z[r]) {
+#pragma unroll
+                for (int e = 0; e < EPW; ++e) {
+                    acc[e][r].x += v[e].x;
+                    acc[e][r].z += v[e].y;
+                }
+            } else {
+                const double2 w = __ldg(ph + (size_t)(r0 + r) * V3 + s);
+#pragma unroll
+                for (int e = 0; e < EPW; ++e) {
+                    acc[e][r].x = ::fma(w.x, v[e].x, acc[e][r].x);
+                    acc[e][r].y = ::fma(w.y, v[e].y, acc[e][r].y);
+                    acc[e][r].z = ::fma(w.x, v[e].y, acc[e][r].z);
+                    acc[e][r].w = ::fma(w.y, v[e].x, acc[e][r].w);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < EPW; ++e)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            if (r0 + r >= n_rep) break;
+            FourierSum &a = acc[e][r];
+#pragma unroll
+            for (int off = 16; off >= 1; off >>= 1) {
+                a.x += __shfl_xor_sync(0xffffffffu, a.x, off);
+                a.z += __shfl_xor_sync(0xffffffffu, a.z, off);
+                if (!z[r]) {
+                    a.y += __shfl_xor_sync(0xffffffffu, a.y, off);
+                    a.w += __shfl_xor_sync(0xffffffffu, a.w, off);
+                }
+            }
+            if (lane == 0 && row + e < rows) out[(size_t)(row + e) * n_rep + r0 + r] = a;
+        }
+}
+// sum of e^{-i p.x} z (CONJ: of e^{-i p.x} conj(z)) from the four sums; sg = -1: at -p.
+template <bool CONJ> __device__ __forceinline__ double2 fourier_value(FourierSum f, int sg) {
+    const double s = sg < 0 ? -1.0 : 1.0;
+    return CONJ ? make_double2(f.x + s * f.y, s * f.w - f.z) : make_double2(f.x - s * f.y, f.z + s * f.w);
 }
 
 // L_Gamma(p, t) = sum_{alpha beta} Gamma_{alpha beta} S_{beta alpha}(p, t):
-// S [n][nt][Q][16] -> out[j][q][G][T] at t = tcol[j] or t_lo + tt.
-static __global__ void mom_gamma_kernel(const double2 *S, const double2 *gammas, int n, int nt, int Q, int T, int t_lo,
-                                        const int *tcol, double2 *out) {
+// F [n][nt][16][n_rep] -> out[j][q][G][T] at t = tcol[j] or t_lo + tt; momentum q is
+// representative rep[q] >> 1, negated if rep[q] & 1.
+static __global__ void mom_gamma_kernel(const FourierSum *F, const double2 *gammas, const int *rep, int n_rep, int n,
+                                        int nt, int Q, int T, int t_lo, const int *tcol, double2 *out) {
     const int total = n * nt * Q * 16;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
         const int G = idx % 16;
         const int q = (idx / 16) % Q;
         const int tt = (idx / (16 * Q)) % nt;
         const int j = idx / (16 * Q * nt);
-        const double2 *s = S + (((size_t)j * nt + tt) * Q + q) * 16;
+        const FourierSum *f = F + ((size_t)j * nt + tt) * 16 * n_rep + (rep[q] >> 1);
+        const int sg = (rep[q] & 1) ? -1 : 1;
         double re = 0.0, im = 0.0;
         for (int al = 0; al < 4; ++al)
             for (int be = 0; be < 4; ++be) {
-                const double2 gm = gammas[(G * 4 + al) * 4 + be], v = s[be * 4 + al];
+                const double2 gm = gammas[(G * 4 + al) * 4 + be];
+                if (gm.x == 0.0 && gm.y == 0.0) continue;
+                const double2 v = fourier_value<false>(f[(size_t)(be * 4 + al) * n_rep], sg);
                 re += gm.x * v.x - gm.y * v.y;
                 im += gm.x * v.y + gm.y * v.x;
             }
@@ -123,72 +295,114 @@ static __global__ void mom_gamma_kernel(const double2 *S, const double2 *gammas,
     }
 }
 
-// Per site of the point-source propagator (canonical [12][V][4][3], column
-// j = 3 alpha + a): P_{(beta alpha),(beta' alpha')} = sum_{a,b}
-// conj(S_{beta b, alpha a}) S_{beta' b, alpha' a}.  One thread per (site, beta,
-// beta'); out [V][256] with V in lexicographic order (t slowest).
-static __global__ void meson_site_kernel(const double *prop, long V, double2 *out) {
-    const long total = V * 16;
-    for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-        const int bb = (int)(idx % 16);
-        const long i = idx / 16;
-        const int be = bb / 4, be2 = bb % 4;
-        cx<double> acc[16];
+// The point-source propagator's products P_{(beta alpha),(beta' alpha')}(x) =
+// sum_{a,b} conj(S_{beta b, alpha a}) S_{beta' b, alpha' a} form a hermitian 16 x 16
+// matrix: 136 entries (beta, alpha) <= (beta', alpha').  Entry number: 40 of the
+// diagonal blocks beta = beta' (10 each), then 6 blocks beta < beta' of 16.
+constexpr int MESON_E = 136;
+__host__ __device__ __forceinline__ int meson_entry(int be, int al, int be2, int al2) {  // (be, al) <= (be2, al2)
+    if (be == be2) return be * 10 + al * 4 - al * (al - 1) / 2 + (al2 - al);
+    return 40 + (be * (7 - be) / 2 + (be2 - be - 1)) * 16 + al * 4 + al2;
+}
+
+// prop: canonical [12][V][4][3], column j = 3 alpha + a; out [t][136][V3].  A block
+// stages the 144 components of 32 sites in shared memory (one contiguous run a
+// column) and gives each of its ten warps one block (beta, beta') of the matrix, a
+// lane per site.  Bound by FP64 (4896 FMA a site, 1.0 ms on 16^3 x 32; all 256
+// entries took 1.95 ms): the hermitian half is all that is formed, and stored
+// entry-major so that lanes write, and the Fourier sums read, contiguous sites.
+static __global__ void __launch_bounds__(320) meson_site_kernel(const double2 *prop, int V, int V3, double2 *out) {
+    extern __shared__ double2 msm[];  // [144][33]
+    const int s0 = blockIdx.x * 32, ns = min(32, V - s0);
+    for (int k = threadIdx.x; k < 12 * 384; k += 320) {
+        const int col = k / 384, e = k - col * 384, site = e / 12, c = e - site * 12;
+        if (site < ns) msm[(col * 12 + c) * 33 + site] = __ldg(prop + ((size_t)col * V + s0) * 12 + e);
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (lane >= ns) return;
+    const int i = s0 + lane;
+    double2 *o = out + (size_t)(i / V3) * MESON_E * V3 + i % V3;
+    auto S = [&](int be, int b, int al, int a) {
+        const double2 v = msm[((3 * al + a) * 12 + 3 * be + b) * 33 + lane];
+        return mk(v.x, v.y);
+    };
+    cx<double> acc[16];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) acc[k] = zero<double>();
-        for (int a = 0; a < 3; ++a) {
-            cx<double> u[4][3], v[4][3];
+    for (int k = 0; k < 16; ++k) acc[k] = zero<double>();
+    if (w < 4) {
+        for (int ab = 0; ab < 9; ++ab) {
+            const int a = ab / 3, b = ab % 3;
+            cx<double> u[4];
+#pragma unroll
+            for (int al = 0; al < 4; ++al) u[al] = S(w, b, al, a);
 #pragma unroll
             for (int al = 0; al < 4; ++al)
 #pragma unroll
-                for (int b = 0; b < 3; ++b) {
-                    const double *pu = prop + (((size_t)(3 * al + a) * V + i) * 12 + be * 3 + b) * 2;
-                    const double *pv = prop + (((size_t)(3 * al + a) * V + i) * 12 + be2 * 3 + b) * 2;
-                    u[al][b] = mk(__ldg(pu), __ldg(pu + 1));
-                    v[al][b] = mk(__ldg(pv), __ldg(pv + 1));
-                }
-#pragma unroll
-            for (int al = 0; al < 4; ++al)
-#pragma unroll
-                for (int al2 = 0; al2 < 4; ++al2)
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) cjmac(acc[al * 4 + al2], u[al][b], v[al2][b]);
+                for (int al2 = al; al2 < 4; ++al2) cjmac(acc[al * 4 + al2], u[al], u[al2]);
         }
-        double2 *o = out + (size_t)i * 256;
 #pragma unroll
         for (int al = 0; al < 4; ++al)
 #pragma unroll
-            for (int al2 = 0; al2 < 4; ++al2)
-                o[(be * 4 + al) * 16 + be2 * 4 + al2] = make_double2(acc[al * 4 + al2].re, acc[al * 4 + al2].im);
+            for (int al2 = al; al2 < 4; ++al2)
+                o[(size_t)meson_entry(w, al, w, al2) * V3] = make_double2(acc[al * 4 + al2].re, acc[al * 4 + al2].im);
+    } else {
+        const int p = w - 4, be = p < 3 ? 0 : (p < 5 ? 1 : 2), be2 = p < 3 ? p + 1 : (p < 5 ? p - 1 : 3);
+        for (int ab = 0; ab < 9; ++ab) {
+            const int a = ab / 3, b = ab % 3;
+            cx<double> u[4], v[4];
+#pragma unroll
+            for (int al = 0; al < 4; ++al) {
+                u[al] = S(be, b, al, a);
+                v[al] = S(be2, b, al, a);
+            }
+#pragma unroll
+            for (int al = 0; al < 4; ++al)
+#pragma unroll
+                for (int al2 = 0; al2 < 4; ++al2) cjmac(acc[al * 4 + al2], u[al], v[al2]);
+        }
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            o[(size_t)meson_entry(be, k / 4, be2, k % 4) * V3] = make_double2(acc[k].re, acc[k].im);
     }
 }
 
 // C^{BA}(q, t - t_src) = - sum g5_alpha g5_beta (Gamma_B)_{beta beta'} (Gamma_A)_{alpha' alpha}
-//                          F_t[q][(beta alpha),(beta' alpha')];  F [T][Q][256], out [Q][16 A][16 B][T].
-static __global__ void meson_gamma_kernel(const double2 *F, const double2 *gammas, int T, int Q, int t_src,
-                                          double2 *out) {
+//                          F_t[q][(beta alpha),(beta' alpha')];  F [T][136][n_rep], out [Q][16 A][16 B][T].
+// Every Gamma of the basis has one non-zero entry per row (its column and value
+// are looked up once per block), so an output is a sum of 16 terms.
+static __global__ void __launch_bounds__(256) meson_gamma_kernel(const FourierSum *F, const double2 *gammas, const int *rep,
+                                                                 int n_rep, int T, int Q, int t_src, double2 *out) {
+    __shared__ double2 val[16][4];
+    __shared__ int col[16][4];
+    for (int k = threadIdx.x; k < 64; k += blockDim.x) {
+        int c = 0;
+        for (int m = 1; m < 4; ++m)
+            if (gammas[k * 4 + m].x != 0.0 || gammas[k * 4 + m].y != 0.0) c = m;
+        col[k / 4][k % 4] = c;
+        val[k / 4][k % 4] = gammas[k * 4 + c];
+    }
+    __syncthreads();
     const int total = Q * 256 * T;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
         const int t = idx % T;
         const int B = (idx / T) % 16;
         const int A = (idx / (16 * T)) % 16;
         const int q = idx / (256 * T);
-        const double2 *f = F + ((size_t)t * Q + q) * 256;
+        const FourierSum *f = F + (size_t)t * MESON_E * n_rep + (rep[q] >> 1);
+        const int sg = (rep[q] & 1) ? -1 : 1;
         double re = 0.0, im = 0.0;
         for (int be = 0; be < 4; ++be)
-            for (int be2 = 0; be2 < 4; ++be2) {
-                const double2 gb = gammas[(B * 4 + be) * 4 + be2];
-                if (gb.x == 0.0 && gb.y == 0.0) continue;
-                for (int al2 = 0; al2 < 4; ++al2)
-                    for (int al = 0; al < 4; ++al) {
-                        const double2 ga = gammas[(A * 4 + al2) * 4 + al];
-                        if (ga.x == 0.0 && ga.y == 0.0) continue;
-                        const double sg = ((al < 2) == (be < 2)) ? 1.0 : -1.0;  // g5_alpha g5_beta
-                        const double2 g = make_double2(sg * (gb.x * ga.x - gb.y * ga.y), sg * (gb.x * ga.y + gb.y * ga.x));
-                        const double2 v = f[(be * 4 + al) * 16 + be2 * 4 + al2];
-                        re += g.x * v.x - g.y * v.y;
-                        im += g.x * v.y + g.y * v.x;
-                    }
+            for (int al2 = 0; al2 < 4; ++al2) {
+                const int be2 = col[B][be], al = col[A][al2];
+                const double2 gb = val[B][be], ga = val[A][al2];
+                const double sn = ((al < 2) == (be < 2)) ? 1.0 : -1.0;  // g5_alpha g5_beta
+                const double2 g = make_double2(sn * (gb.x * ga.x - gb.y * ga.y), sn * (gb.x * ga.y + gb.y * ga.x));
+                const bool lower = be * 4 + al > be2 * 4 + al2;
+                const double2 v = lower ? fourier_value<true>(f[(size_t)meson_entry(be2, al2, be, al) * n_rep], sg)
+                                        : fourier_value<false>(f[(size_t)meson_entry(be, al, be2, al2) * n_rep], sg);
+                re += g.x * v.x - g.y * v.y;
+                im += g.x * v.y + g.y * v.x;
             }
         out[(((size_t)q * 16 + A) * 16 + B) * T + (t - t_src + T) % T] = make_double2(-re, -im);
     }
