@@ -127,6 +127,8 @@ struct dl_ctx {
     };
     Scratch s_phase, s_site, s_msum, s_mloops, s_mgroup, s_mom, s_cover, s_out;
 
+    SmearList *d_smear = nullptr;  // columns and groups of the current smearing
+
     int *h_count = nullptr;  // pinned, mapped
     int *d_count = nullptr;
 
@@ -753,6 +755,7 @@ extern "C" int dl_create(dl_ctx **out, const int dims[4], int t_bc, void *cuda_s
         cudaMalloc((void **)&c->d_gammas, 256 * sizeof(double2)) != cudaSuccess ||
         cudaMalloc((void **)&c->d_acc, 2 * 16 * dims[3] * sizeof(double2)) != cudaSuccess ||
         cudaMalloc((void **)&c->d_tcol, 128 * sizeof(int)) != cudaSuccess ||
+        cudaMalloc((void **)&c->d_smear, sizeof(SmearList)) != cudaSuccess ||
         cudaMalloc((void **)&c->d_acc2, (size_t)64 * 2 * 16 * dims[3] * sizeof(double2)) != cudaSuccess ||
         cudaHostAlloc((void **)&c->h_count, sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer((void **)&c->d_count, c->h_count, 0) != cudaSuccess ||
@@ -784,6 +787,7 @@ extern "C" int dl_destroy(dl_ctx *c) {
     void *ptrs[] = {c->d_coords,   c->d_gauge64, c->d_gauge32,  c->d_gauge16, c->d_gauge8_32, c->d_gauge8_16, c->d_gauge8q,
                     c->d_gauge8d,
                     c->d_gauge_ff, c->d_gammas,  c->d_partials, c->d_acc,     c->d_noise,     c->d_w,
+                    c->d_smear,
                     c->d_reslinks[0], c->d_reslinks[1], c->d_reslinks[2],
                     c->d_tcol,     c->d_acc2,    c->d_clov64,   c->d_clovinv64, c->d_clovinv32, c->d_clovinv16};
     for (void *p : ptrs)
@@ -1732,26 +1736,34 @@ static int smear_eo(dl_ctx *c, double **buf, double *spare, int N, int n, const 
     } else {
         double *src2 = buf2 ? *buf2 : nullptr, *dst2 = spare2;
         const int nf = buf2 ? 2 : 1;
+        SmearList *L = c->d_smear;
+        CK(cudaMemsetAsync(L, 0, offsetof(SmearList, g), c->cur));
+        Launch lf = make_launch(c, 2L * (cb1 - cb0) * n, 256, 0, 8);
         Launch lc = make_launch(c, 2L * (cb1 - cb0) * 12 * n, 256, 0, 8);
-        ff_convert_kernel<<<lc.grid, lc.block, 0, c->cur>>>(src, (int)c->Vh, cb0, cb1, N, n, 1, tcol, c->g.V3h);
-        if (buf2)
-            ff_convert_kernel<<<lc.grid, lc.block, 0, c->cur>>>(src2, (int)c->Vh, cb0, cb1, N, n, 1, tcol, c->g.V3h);
-        // one thread per (site, colour row, column): three times the threads of
-        // the whole-site kernel, each with a third of the registers
-        Launch lr = make_launch(c, 2L * (cb1 - cb0) * 3 * n, 256, 0, 6);
+        for (int f = 0; f < nf; ++f) {
+            double *x = f ? src2 : src;
+            smear_flags_kernel<<<lf.grid, lf.block, 0, c->cur>>>(x, (int)c->Vh, cb0, cb1, N, n, tcol, c->g.V3h,
+                                                                 L->flags[f]);
+            ff_convert_kernel<<<lc.grid, lc.block, 0, c->cur>>>(x, (int)c->Vh, cb0, cb1, N, n, 1, tcol, c->g.V3h,
+                                                                nullptr);
+        }
+        smear_list_kernel<<<1, 64, 0, c->cur>>>(L, n, nf, tcol);
+        // one thread per (site, colour row, group of columns), sized for dense fields; the
+        // list's length is known on the device only
+        Launch lr = make_launch(c, 2L * (cb1 - cb0) * 3 * n * nf, 256, 0, 64);
         for (int it = 0; it < s.n_iter; ++it) {
             A.in = src;
             A.out = dst;
             A.in2 = src2;
             A.out2 = dst2;
-            smear_ff_rows_kernel<<<dim3(lr.grid, nf), lr.block, 0, c->cur>>>(A, c->d_gauge_ff);
+            smear_ff_rows_kernel<<<lr.grid, lr.block, 0, c->cur>>>(A, c->d_gauge_ff, L);
             std::swap(src, dst);
             std::swap(src2, dst2);
         }
-        ff_convert_kernel<<<lc.grid, lc.block, 0, c->cur>>>(src, (int)c->Vh, cb0, cb1, N, n, 0, tcol, c->g.V3h);
-        if (buf2)
-            ff_convert_kernel<<<lc.grid, lc.block, 0, c->cur>>>(src2, (int)c->Vh, cb0, cb1, N, n, 0, tcol, c->g.V3h);
-        c->kernel_launches += s.n_iter + 2 * nf;
+        for (int f = 0; f < nf; ++f)
+            ff_convert_kernel<<<lc.grid, lc.block, 0, c->cur>>>(f ? src2 : src, (int)c->Vh, cb0, cb1, N, n, 0, tcol,
+                                                                c->g.V3h, &L->flags[f][0][0]);
+        c->kernel_launches += s.n_iter + 3 * nf + 1;
         if (buf2) *buf2 = src2;
     }
     CK(cudaGetLastError());
@@ -1888,7 +1900,7 @@ static int contract_eo(dl_ctx *c, const double *eta, const double *phi, int n, i
     else contract_kernel<2><<<grid, block, smem, c->cur>>>(A);
     const int cnt = n * 16 * T;
     zero_kernel<<<std::max(1, (cnt + 255) / 256), 256, 0, c->cur>>>(dst, cnt);
-    contract_final_kernel<<<dim3(nt, n), 32, 0, c->cur>>>(c->d_partials, nbx, N, t_lo, T, c->d_gammas, dst, tcol);
+    contract_final_kernel<<<dim3(nt, n), 256, 0, c->cur>>>(c->d_partials, nbx, N, t_lo, T, c->d_gammas, dst, tcol);
     c->kernel_launches += 3;
     CK(cudaGetLastError());
     return DL_OK;

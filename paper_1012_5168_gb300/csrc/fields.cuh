@@ -438,8 +438,9 @@ __device__ __forceinline__ ffc ld_ffc(const double *p) {
 
 // In-place conversion of an EO tile field (both parities, cb range, n of N
 // columns) between FP64 and float-float.  to_ff = 1: double -> ff; 0: back.
+// flags (back only): spins flags[j][s] == 0 were left out of the iterations and become 0.
 static __global__ void ff_convert_kernel(double *f, int Vh, int cb0, int cb1, int N, int n, int to_ff,
-                                         const int *tcol, int V3h) {
+                                         const int *tcol, int V3h, const int *flags) {
     const long nsite = cb1 - cb0;
     const long total = 2 * nsite * 12 * n;
     for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
@@ -457,8 +458,9 @@ static __global__ void ff_convert_kernel(double *f, int Vh, int cb0, int cb1, in
             const float4 v = *reinterpret_cast<const float4 *>(e);
             ff a, b;
             a.hi = v.x; a.lo = v.y; b.hi = v.z; b.lo = v.w;
-            e[0] = (double)a;
-            e[1] = (double)b;
+            const bool on = flags[j * 4 + c / 3] != 0;
+            e[0] = on ? (double)a : 0.0;
+            e[1] = on ? (double)b : 0.0;
         }
     }
 }
@@ -471,29 +473,115 @@ static __global__ void gauge_ff_kernel(const double *g64, float *out, long n_com
     }
 }
 
+// Smearing acts on each spin of a field by itself (the links are colour
+// matrices), and K 0 = 0: a spin-diluted source has three spins without work.
+// The columns (field, right-hand side, spin) that hold a non-zero value are
+// flagged from the fields themselves and gathered in groups of four of one field
+// and one timeslice; a thread smears one group, with one load of the link row.  A
+// dense right-hand side is one group, its four spins.
+struct SmearGroup {
+    int field;   // 0: in/out, 1: in2/out2
+    int t;       // timeslice (with tcol), else 0
+    int col[4];  // right-hand side << 2 | spin, or -1
+};
+struct SmearList {
+    int n_groups;
+    int flags[2][64][4];
+    SmearGroup g[128];
+};
+
+// flags of one field (cleared before): blocks over sites, right-hand sides fastest.
+static __global__ void smear_flags_kernel(const double *f, int Vh, int cb0, int cb1, int N, int n, const int *tcol,
+                                          int V3h, int (*flags)[4]) {
+    const long nsite = cb1 - cb0, total = 2 * nsite * n;
+    for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
+        const int j = (int)(idx % n);
+        const long sp = idx / n;
+        const int p = (int)(sp / nsite);
+        const int cb = cb0 + (int)(sp % nsite) + (tcol ? tcol[j] * V3h : 0);
+        const uint4 *e = reinterpret_cast<const uint4 *>(f) + ((size_t)p * Vh + cb) * 12 * N + j;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            unsigned any = 0;
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                const uint4 v = __ldg(e + (size_t)(3 * s + b) * N);
+                any |= v.x | (v.y << 1) | v.z | (v.w << 1);  // (the sign bits do not count)
+            }
+            if (any && ((volatile int *)flags[j])[s] == 0) ((volatile int *)flags[j])[s] = 1;
+        }
+    }
+}
+
+// One block of 64 threads: groups of each field in the order of its right-hand sides.
+static __global__ void smear_list_kernel(SmearList *L, int n, int nf, const int *tcol) {
+    __shared__ int flags[2][64][4], ts[64], count[2];
+    __shared__ SmearGroup g[2][64];
+    for (int k = threadIdx.x; k < 512; k += 64) flags[k >> 8][(k >> 2) & 63][k & 3] = L->flags[k >> 8][(k >> 2) & 63][k & 3];
+    if ((int)threadIdx.x < n) ts[threadIdx.x] = tcol ? tcol[threadIdx.x] : 0;
+    __syncthreads();
+    if ((int)threadIdx.x < 2) {
+        const int f = threadIdx.x;
+        int m = 0, k = 0;  // groups; columns in the open group
+        for (int j = 0; j < n && f < nf; ++j) {
+            if (k && g[f][m].t != ts[j]) {
+                ++m;
+                k = 0;
+            }
+            for (int s = 0; s < 4; ++s) {
+                if (!flags[f][j][s]) continue;
+                if (!k) {
+                    g[f][m].field = f;
+                    g[f][m].t = ts[j];
+                    for (int q = 1; q < 4; ++q) g[f][m].col[q] = -1;
+                }
+                g[f][m].col[k] = j << 2 | s;
+                if (++k == 4) {
+                    ++m;
+                    k = 0;
+                }
+            }
+        }
+        count[f] = m + (k ? 1 : 0);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < count[0] + count[1]; k += 64) L->g[k] = k < count[0] ? g[0][k] : g[1][k - count[0]];
+    if (threadIdx.x == 0) L->n_groups = count[0] + count[1];
+}
+
 // One smearing step in float-float (same contract as smear_kernel, fields
-// and links in float-float format), with the three colour rows of a site on
-// three threads: thread (site, a, j) produces the four spin components of
-// colour a.  It holds one link row and one colour vector at a time instead of
-// the whole link and the 12-component accumulator, so it needs far fewer
-// registers and more warps stay resident; the three threads of a site read the
-// same neighbour spinors, which then come from L1.  Two resident blocks per SM
-// (up to 128 registers a thread) measured 9% faster than three (85): 0.198
-// against 0.217 ms per iteration for 96 fields on one 16^3 timeslice.
-static __global__ void __launch_bounds__(256, 2) smear_ff_rows_kernel(SmearArgs A, const float *gauge_ff) {
-    const int nsite = A.cb1 - A.cb0;
-    const long total = 2L * nsite * 3 * A.n;  // only the columns in use
+// and links in float-float format) on the groups of the list, with the three
+// colour rows of a site on three threads: thread (site, a, group) produces colour
+// a of the group's four columns.  It holds one link row and one colour vector at a
+// time instead of the whole link and the 12-component accumulator, so it needs far
+// fewer registers and more warps stay resident; the three threads of a site read
+// the same neighbour spinors, which then come from L1.  Bound by the FP32 units (12
+// instructions a product).  Two resident blocks per SM (up to 128 registers a
+// thread) measured 9% faster than three (85).  48 pairs of spin-diluted sources
+// and solutions on one 16^3 timeslice: 114 us a step with the groups, 176 us
+// on all 384 columns.
+static __global__ void __launch_bounds__(256, 2) smear_ff_rows_kernel(SmearArgs A, const float *gauge_ff,
+                                                                      const SmearList *L) {
+    const int nsite = A.cb1 - A.cb0, ng = L->n_groups;
+    const long total = 2L * nsite * 3 * ng;
     const size_t half = (size_t)A.g.Vh * 12 * A.N * 2;
     const ff fa = df_from_double(A.a), fc = df_from_double(A.c);
-    const double *__restrict__ fin = blockIdx.y ? A.in2 : A.in;  // the field of this grid row
-    double *__restrict__ fout = blockIdx.y ? A.out2 : A.out;
     for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-        const int j = (int)(idx % A.n);
-        const long rest = idx / A.n;
+        const int gi = (int)(idx % ng);
+        const long rest = idx / ng;
         const int a = (int)(rest % 3);
         const int sp = (int)(rest / 3);
         const int p = sp / nsite;
-        const int cb = A.cb0 + sp % nsite + col_offset(A.tcol, j, A.n, A.g);
+        const SmearGroup G = L->g[gi];
+        const double *__restrict__ fin = G.field ? A.in2 : A.in;
+        double *__restrict__ fout = G.field ? A.out2 : A.out;
+        const int cb = A.cb0 + sp % nsite + (A.tcol ? G.t * A.g.V3h : 0);
+        uint32_t off[4];  // offsets of the columns within a site's [12][N] complex (a missing column reads the first)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int col = G.col[k] < 0 ? G.col[0] : G.col[k];
+            off[k] = (uint32_t)(3 * (col & 3) * A.N + (col >> 2)) * 2;
+        }
         const Site st = decode(__ldg(A.coords + (size_t)p * A.g.Vh + cb), A.g);
         const double *inn = fin + (size_t)(1 - p) * half;
         cdacc acc[4];  // unnormalised sums (common.cuh), renormalised once at the end
@@ -514,27 +602,26 @@ static __global__ void __launch_bounds__(256, 2) smear_ff_rows_kernel(SmearArgs 
                     const ffc w = ld_ffc(up + 2 * (dir == 0 ? a * 3 + b : b * 3 + a));
                     u[b] = mk(w.re, w.im);
                 }
-                const double *src = inn + (size_t)nb * 12 * A.N * 2 + (size_t)j * 2;
+                const double *src = inn + (size_t)nb * 12 * A.N * 2;
 #pragma unroll
                 for (int s = 0; s < 4; ++s)
 #pragma unroll
                     for (int b = 0; b < 3; ++b) {
-                        const ffc v = ld_ffc(src + (size_t)(3 * s + b) * A.N * 2);
+                        const ffc v = ld_ffc(src + off[s] + b * A.N * 2);
                         if (dir == 0) cda_mac<false>(acc[s], u[b], mk(v.re, v.im));
                         else cda_mac<true>(acc[s], u[b], mk(v.re, v.im));
                     }
             }
         }
-        const double *y = fin + (size_t)p * half + (size_t)cb * 12 * A.N * 2 + (size_t)j * 2;
-        double *o = fout + (size_t)p * half + (size_t)cb * 12 * A.N * 2 + (size_t)j * 2;
+        const size_t site = (size_t)p * half + (size_t)cb * 12 * A.N * 2 + (size_t)a * A.N * 2;
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-            const int k = 3 * s + a;
-            const ffc q = ld_ffc(y + (size_t)k * A.N * 2);
+            const ffc q = ld_ffc(fin + site + off[s]);
             ffc r;
             r.re = df_add(df_mul(fa, q.re), df_mul(fc, da_norm(acc[s].re)));
             r.im = df_add(df_mul(fa, q.im), df_mul(fc, da_norm(acc[s].im)));
-            *reinterpret_cast<float4 *>(o + (size_t)k * A.N * 2) = make_float4(r.re.hi, r.re.lo, r.im.hi, r.im.lo);
+            if (G.col[s] >= 0)
+                *reinterpret_cast<float4 *>(fout + site + off[s]) = make_float4(r.re.hi, r.re.lo, r.im.hi, r.im.lo);
         }
     }
 }
@@ -598,31 +685,41 @@ static __global__ void __launch_bounds__(128) contract_kernel(ContractArgs A) {
     block_reduce<R, 16, double>(acc, G, A.N, part, smem);
 }
 
-// final: sum partials over (parity, bx) in fixed order, then L_Gamma(t) =
-// sum_{alpha beta} Gamma_{alpha beta} S_{beta alpha}.  out[j][16][T] double2.
-// grid = (n_t, n), block = 32.
-static __global__ void contract_final_kernel(const double2 *partials, int nbx, int N, int t_lo, int T,
+// final: sum partials over (parity, bx) in fixed order (16 runs per value, then the
+// runs: one lane per value took 110 us for 608 blocks, 14 us now), then
+// L_Gamma(t) = sum_{alpha beta} Gamma_{alpha beta} S_{beta alpha}.  out[j][16][T]
+// double2.  grid = (n_t, n), block = 256.
+static __global__ void __launch_bounds__(256) contract_final_kernel(const double2 *partials, int nbx, int N, int t_lo, int T,
                                       const double2 *gammas /* [16][4][4] */, double2 *out, const int *tcol) {
     const int tt = blockIdx.x;
     const int j = blockIdx.y;
-    __shared__ double2 S[16];
-    const int lane = threadIdx.x;
-    if (lane < 16) {
+    __shared__ double2 R[16][16], S[16];
+    const int lane = threadIdx.x & 15, run = threadIdx.x >> 4;
+    {
         double re = 0.0, im = 0.0;
-        for (int p = 0; p < 2; ++p)
-            for (int b = 0; b < nbx; ++b) {
-                const double2 v = partials[(((size_t)(tt * 2 + p) * nbx + b) * N + j) * 16 + lane];
-                re += v.x;
-                im += v.y;
-            }
+        for (int b = run; b < 2 * nbx; b += 16) {  // b = parity * nbx + bx
+            const double2 v = partials[(((size_t)tt * 2 * nbx + b) * N + j) * 16 + lane];
+            re += v.x;
+            im += v.y;
+        }
+        R[run][lane] = make_double2(re, im);
+    }
+    __syncthreads();
+    if (threadIdx.x < 16) {
+        double re = 0.0, im = 0.0;
+        for (int k = 0; k < 16; ++k) {
+            re += R[k][lane].x;
+            im += R[k][lane].y;
+        }
         S[lane] = make_double2(re, im);  // S[beta*4 + alpha]
     }
     __syncthreads();
-    if (lane < 16) {
+    if (threadIdx.x < 16) {
         double re = 0.0, im = 0.0;
         for (int al = 0; al < 4; ++al)
             for (int be = 0; be < 4; ++be) {
                 const double2 gm = gammas[(lane * 4 + al) * 4 + be];
+                if (gm.x == 0.0 && gm.y == 0.0) continue;
                 const double2 s = S[be * 4 + al];
                 re += gm.x * s.x - gm.y * s.y;
                 im += gm.x * s.y + gm.y * s.x;
