@@ -64,6 +64,12 @@ __device__ __forceinline__ void cjmac(cx<T> &acc, cx<T> a, cx<T> b) {
     acc.im = fma(a.re, b.im, acc.im);
     acc.im = fma(-a.im, b.re, acc.im);
 }
+// acc += |a|^2 (the real part of conj(a) a, summed as cjmac does; the imaginary part stays 0)
+template <typename T>
+__device__ __forceinline__ void norm_mac(cx<T> &acc, cx<T> a) {
+    acc.re = fma(a.re, a.re, acc.re);
+    acc.re = fma(a.im, a.im, acc.re);
+}
 template <typename T>
 __device__ __forceinline__ cx<T> zero() { return mk<T>(T(0), T(0)); }
 

@@ -277,6 +277,83 @@ __device__ __forceinline__ void hop_dir_x2(const HopArgs &A, const Site &st, int
     reconstruct_x2<MU, SG>(w, acc);
 }
 
+// w += U h (DAG: U^dag h): the products continue the sums already in w.
+template <typename T, bool DAG>
+__device__ __forceinline__ void su3_mac(const cx<T> (&u)[9], const cx<T> (&h)[6], cx<T> (&w)[6]) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                if (DAG) cjmac(w[3 * s + a], u[b * 3 + a], h[3 * s + b]);
+                else cmac(w[3 * s + a], u[a * 3 + b], h[3 * s + b]);
+            }
+}
+
+// Both directions of mu for FP64, which is bound by the FP64 units (two FMA lanes
+// a clock and SM), in fewer instructions: with w+ = U h+ and w- = U^dag h- the
+// spins get [w+ + w-; X^dag (w- - w+)].  The products of w- continue the sums of
+// w+ (A = w+ + w-, no additions), B = A - 2 w+ is one FMA, and A and B are added
+// once where w+ and w- were added twice: 204 FP64 instructions instead of 216, the
+// first mu (FIRST) starts the sums instead of adding to zeros.
+template <int MU, bool FIRST>
+__device__ __forceinline__ void hop_pair_f64(const HopArgs &A, const Site &st, int cb, int r0, cx<double> (&acc)[12]) {
+    const double *in = reinterpret_cast<const double *>(A.in);
+    const double *gauge = reinterpret_cast<const double *>(A.gauge);
+    const size_t N = (size_t)A.N;
+    cx<double> w[6], a[6];
+#pragma unroll
+    for (int dir = 0; dir < 2; ++dir) {
+        const int nb = dir == 0 ? nbr_fwd(st, A.g, MU) : nbr_bwd(st, A.g, MU);
+        const double *up = dir == 0 ? gauge + (((size_t)A.p * A.g.Vh + cb) * 4 + MU) * 18
+                                    : gauge + (((size_t)(1 - A.p) * A.g.Vh + nb) * 4 + MU) * 18;
+        cx<double> u[9], h[1][6];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) u[k] = ld_link<double>(up + 2 * k);
+        const double *src = in + (size_t)nb * 12 * N * 2 + (size_t)r0 * 2;
+        if (dir == 0) load_project<double, 1, MU, -1>(src, N, h);
+        else load_project<double, 1, MU, +1>(src, N, h);
+        if (MU == 3 && A.g.t_bc < 0 && st.c[3] == (dir == 0 ? A.g.L[3] - 1 : 0)) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {  // a sign flip by the sign bit
+                h[0][k].re = __hiloint2double(__double2hiint(h[0][k].re) ^ (int)0x80000000, __double2loint(h[0][k].re));
+                h[0][k].im = __hiloint2double(__double2hiint(h[0][k].im) ^ (int)0x80000000, __double2loint(h[0][k].im));
+            }
+        }
+        if (dir == 0) {
+            su3_mul<double, false>(u, h[0], w);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) a[k] = w[k];
+        } else {
+            su3_mac<double, true>(u, h[0], a);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        w[k] = mk(::fma(-2.0, w[k].re, a[k].re), ::fma(-2.0, w[k].im, a[k].im));  // w- - w+
+        acc[k] = FIRST ? a[k] : acc[k] + a[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const cx<double> b0 = w[k], b1 = w[3 + k];
+        cx<double> &l0 = acc[6 + k], &l1 = acc[9 + k];
+        if (MU == 0) {  // X^dag b = (-i b1, -i b0)
+            l0 = FIRST ? tmi(b1) : l0 + tmi(b1);
+            l1 = FIRST ? tmi(b0) : l1 + tmi(b0);
+        } else if (MU == 1) {  // (b1, -b0)
+            l0 = l0 + b1;
+            l1 = l1 - b0;
+        } else if (MU == 2) {  // (-i b0, i b1)
+            l0 = l0 + tmi(b0);
+            l1 = l1 + ti(b1);
+        } else {
+            l0 = l0 + b0;
+            l1 = l1 + b1;
+        }
+    }
+}
+
 // NC > 0: the number of right-hand sides in the layout is the compile-time
 // constant NC (= A.N), so component offsets fold into the load and store
 // instructions; NC = 0 reads it from A.N.
@@ -339,14 +416,21 @@ __device__ __forceinline__ void hop_body(const HopArgs &A) {
 #pragma unroll
             for (int c = 0; c < 12; ++c) acc[0][c] = mk((T)a2[c].x, (T)a2[c].y);
         } else {
+            if constexpr (sizeof(S) == 8) {
+                hop_pair_f64<0, true>(A, st, cb, r0, acc[0]);
+                hop_pair_f64<1, false>(A, st, cb, r0, acc[0]);
+                hop_pair_f64<2, false>(A, st, cb, r0, acc[0]);
+                hop_pair_f64<3, false>(A, st, cb, r0, acc[0]);
+            } else {
 #pragma unroll
-            for (int r = 0; r < R; ++r)
+                for (int r = 0; r < R; ++r)
 #pragma unroll
-                for (int c = 0; c < 12; ++c) acc[r][c] = zero<T>();
-            hop_dir<S, R, 0, NC>(A, st, cb, r0, acc);
-            hop_dir<S, R, 1, NC>(A, st, cb, r0, acc);
-            hop_dir<S, R, 2, NC>(A, st, cb, r0, acc);
-            hop_dir<S, R, 3, NC>(A, st, cb, r0, acc);
+                    for (int c = 0; c < 12; ++c) acc[r][c] = zero<T>();
+                hop_dir<S, R, 0, NC>(A, st, cb, r0, acc);
+                hop_dir<S, R, 1, NC>(A, st, cb, r0, acc);
+                hop_dir<S, R, 2, NC>(A, st, cb, r0, acc);
+                hop_dir<S, R, 3, NC>(A, st, cb, r0, acc);
+            }
             if constexpr (CLOV != 0 && R == 1)  // clover: A^-1 of the output site on D in
                 clover_inv_apply<S, T>(reinterpret_cast<const S *>(A.clovinv) + ((size_t)A.p * A.g.Vh + cb) * 72 * 2,
                                        acc[0]);
@@ -358,9 +442,9 @@ __device__ __forceinline__ void hop_body(const HopArgs &A) {
         for (int c = 0; c < 12; ++c) {
             const size_t off = base + (size_t)c * N * 2;
             cx<T> o[R];
-            if (MODE == MODE_PLAIN) {
+            if (MODE == MODE_PLAIN) {  // (an FP64 product by one is as dear as any)
 #pragma unroll
-                for (int r = 0; r < R; ++r) o[r] = cD * acc[r][c];
+                for (int r = 0; r < R; ++r) o[r] = sizeof(S) == 8 && A.c == 1.0 ? acc[r][c] : cD * acc[r][c];
             }
             cx<T> yv[R];
             if (MODE == MODE_XPAY || MODE == MODE_RESID || RED == RED_BICG) {
@@ -385,15 +469,15 @@ __device__ __forceinline__ void hop_body(const HopArgs &A) {
                         cjmac(red[r][0], rh[r], o[r]);
                     } else {
                         cjmac(red[r][0], o[r], yv[r]);   // <t, s>
-                        cjmac(red[r][1], o[r], o[r]);    // <t, t>
+                        norm_mac(red[r][1], o[r]);       // <t, t>
                         cjmac(red[r][2], rh[r], yv[r]);  // <rhat, s>
                         cjmac(red[r][3], rh[r], o[r]);   // <rhat, t>
-                        cjmac(red[r][4], yv[r], yv[r]);  // <s, s>
+                        norm_mac(red[r][4], yv[r]);      // <s, s>
                     }
                 }
             } else if (RED == RED_NORM) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) cjmac(red[r][0], o[r], o[r]);
+                for (int r = 0; r < R; ++r) norm_mac(red[r][0], o[r]);
             }
         }
     }

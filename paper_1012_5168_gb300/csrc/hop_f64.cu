@@ -1,6 +1,7 @@
 // Wilson-hop instantiations for double storage: FP64 arithmetic, and float-float
 // arithmetic (hop_ff.cuh) for the defect-correction steps of mixed-precision solves.
 #include "hop_ff.cuh"
+#include "hop_split.cuh"
 #include "launch.h"
 
 namespace dl {
@@ -12,8 +13,25 @@ static cudaError_t go(const HopArgs &a, Launch &l) {
         hop_kernel_clov<double, MODE, RED><<<l.grid, l.block, l.smem, l.stream>>>(a);
         return cudaGetLastError();
     }
-    clamp_grid(l, resident_blocks(hop_kernel<double, R, MODE, RED>, l.block, l.smem));
-    hop_kernel<double, R, MODE, RED><<<l.grid, l.block, l.smem, l.stream>>>(a);
+    // Where every SM gets at most one block of 64 (site, right-hand side) items, four warps
+    // share 32 of them (hop_split.cuh), one group a block while that fills no more than the
+    // SMs: plain hops of 12.4 us (up to 32 items an SM) and 18.5 us (64) against 31 us for
+    // any number of sites up to 100 an SM; at 108 items an SM both take 33 us.
+    const long items = (long)(a.cb_end - a.cb_begin) * a.N;
+    if (l.num_sms > 0 && items <= 64L * l.num_sms) {
+        const int groups = a.N <= 32 && items <= 32L * l.num_sms ? 1 : 2;
+        auto kernel = groups == 1 ? hop_split_f64_kernel<MODE, RED, 1> : hop_split_f64_kernel<MODE, RED, 2>;
+        l.block = 128 * groups;
+        l.smem = 0;
+        l.grid = (int)((items + 32 * groups - 1) / (32 * groups));
+        kernel<<<l.grid, l.block, 0, l.stream>>>(a);
+        return cudaGetLastError();
+    }
+    // 168 registers let six blocks of 64 threads share an SM (about 180: five).  One right-hand
+    // side on 16^3 x 32: 107 / 115 / 135 us (plain, <rhat, v>, five sums) against 116 / 125 / 144.
+    auto kernel = hop_kernel_cap<double, R, MODE, RED, 168>;
+    clamp_grid(l, resident_blocks(kernel, l.block, l.smem));
+    kernel<<<l.grid, l.block, l.smem, l.stream>>>(a);
     return cudaGetLastError();
 }
 

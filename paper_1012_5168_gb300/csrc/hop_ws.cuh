@@ -182,15 +182,15 @@ __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
                         cjmac(red[r][0], rh[r], o[r]);
                     } else {
                         cjmac(red[r][0], o[r], yv[r]);
-                        cjmac(red[r][1], o[r], o[r]);
+                        norm_mac(red[r][1], o[r]);
                         cjmac(red[r][2], rh[r], yv[r]);
                         cjmac(red[r][3], rh[r], o[r]);
-                        cjmac(red[r][4], yv[r], yv[r]);
+                        norm_mac(red[r][4], yv[r]);
                     }
                 }
             } else if (RED == RED_NORM) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) cjmac(red[r][0], o[r], o[r]);
+                for (int r = 0; r < R; ++r) norm_mac(red[r][0], o[r]);
             }
         }
     }
