@@ -45,7 +45,8 @@ HOP_KIND_NAMES = {0: "hop_kernel_cap (direct)", 1: "hop_kernel_pf (cp.async pref
                   4: "hop_kernel_ws (warp-staged)", 5: "hop_kernel_mma (tensor cores)",
                   6: "hop_kernel_x2 (packed FP32)", 7: "hop_kernel_pair (paired layout)",
                   8: "hop_kernel_pair_cap (paired layout)", 9: "hop_kernel_ws_pair (paired, warp-staged)",
-                  10: "hop_kernel_cap (direct, wider register cap)", 11: "hop_kernel_ws (warp-staged, two stages)"}
+                  10: "hop_kernel_cap (direct, wider register cap)", 11: "hop_kernel_ws (warp-staged, two stages)",
+                  12: "hop_kernel_ws (warp-staged, two sites per warp)"}
 
 
 def parse():

@@ -434,15 +434,18 @@ int dl_bench_hop(dl_ctx *ctx, int precision, int n_rhs, int fused, int reps,
  * (DLOOPS_F32_PAIRS=1, even widths) 0, 7 and 8 (packed, uncapped and capped)
  * and 9 (packed, warp-staged; widths 32 and 64); 10 the direct FP32 kernel
  * under a wider register cap (R = 1); 11 warp-staged with two stages per warp
- * (widths 32 R, twice the warps per SM of kind 4).  Each candidate times three classes of
+ * (widths 32 R, twice the warps per SM of kind 4); 12 the same at width 16 with two
+ * sites per warp (FP32, R = 1).  Each candidate times three classes of
  * hops on random fields: the plain hop (class 0), the fused hop with <rhat, v>
  * (class 1, which also serves the other fused hops) and the fused hop with the
- * five BiCGStab reductions (class 2), in two sweeps over all candidates, and
- * the fastest is kept for each class separately (so they may use different
+ * five BiCGStab reductions (class 2), once for every candidate and twice more for
+ * those near the fastest, and the fastest is kept for each class separately (so they may use different
  * kernels); another kind replaces the direct kernel only when it is more than
  * 2% faster.  force_R / force_block > 0 and force_pf >= 0 restrict the
- * candidates (for all classes).  Solves tune their (precision, batch) on first
- * use.  *R_out, *block_out, *pf_out receive the class-2 choice and *ms_out the
+ * candidates (for all classes) and pin the width: its solves then run step by step
+ * with these kernels, where a small lattice would otherwise run its inner phases in
+ * one launch.  Step-by-step FP32 and BF16 solves tune their (precision, batch) on
+ * first use.  *R_out, *block_out, *pf_out receive the class-2 choice and *ms_out the
  * time of one plain plus one class-2 hop (each may be NULL).  The call
  * overwrites the context's inner workspace, so make it between solves.
  * Errors: DL_EINVAL (arguments, or a kind the storage layout lacks),
@@ -456,8 +459,8 @@ int dl_tune_hop(dl_ctx *ctx, int precision, int n_rhs, int force_R, int force_bl
  * be NULL).  No tuning, no GPU work.  Errors: DL_EINVAL. */
 int dl_hop_shape(dl_ctx *ctx, int precision, int n_rhs, int cls, int *R_out, int *block_out, int *kind_out);
 /* Set that launch shape explicitly (R in {1, 2, 4}, block in {64, 128, 256},
- * kind as dl_tune_hop; kinds 3-5, 9 and 11 take block 64 and size their own
- * blocks); the width then counts as tuned.  Errors: DL_EINVAL for a shape the
+ * kind 0-11 as dl_tune_hop; kinds 3-5, 9 and 11 take block 64 and size their own
+ * blocks); the width then counts as tuned and pinned.  Errors: DL_EINVAL for a shape the
  * precision, width or storage layout does not allow. */
 int dl_set_hop_shape(dl_ctx *ctx, int precision, int n_rhs, int cls, int R, int block, int kind);
 

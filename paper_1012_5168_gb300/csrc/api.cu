@@ -147,7 +147,8 @@ struct dl_ctx {
     int hop_kind[5][8][3];   // 0 direct, 1 cp.async prefetching, 2 bulk-copy staged, 3 blocked, 4 warp-staged,
                           // 5 tensor cores (BF16), 6 direct with packed FP32 arithmetic, 7 paired layout with
                           // packed FP32 arithmetic, 8 the same under a 128-register cap, 9 paired and
-                          // warp-staged, 10 direct under a wider register cap, 11 warp-staged with two stages
+                          // warp-staged, 10 direct under a wider register cap, 11 warp-staged with two stages,
+                          // 12 the same at width 16 with two sites per warp (the tuner's choice only)
     bool hop_tuned[5][8];
     bool hop_pinned[5][8];   // shapes forced by the caller: solves of that width keep to them (no resident solver)
     // cluster-resident solver: its links per storage precision, stale after a change of the links
@@ -470,7 +471,8 @@ static int time_hops(dl_ctx *c, int prec, int N, int reps, float *ms_out, int wh
 // right-hand sides per thread and B threads per block (bi: B's index in
 // {64, 128, 256}).
 static bool shape_ok(int prec, int N, int R, int B, int bi, int pf) {
-    if (pf < 0 || pf > 11 || (prec == P_F64 && (pf != 0 || R != 1))) return false;
+    if (pf < 0 || pf > 12 || (prec == P_F64 && (pf != 0 || R != 1))) return false;
+    if (pf == 12) return prec == P_F32 && R == 1 && N == 16 && bi == 0;
     if (pf == 10 && (prec != P_F32 || R != 1)) return false;       // wider-cap direct: FP32, one per thread
     if (prec == P_F32P ? (pf != 0 && (pf < 7 || pf > 9)) : (pf >= 7 && pf <= 9)) return false;  // paired: 0, 7-9
     if (pf == 11 && prec == P_F32P) return false;
@@ -493,50 +495,56 @@ static int tune_hop(dl_ctx *c, int prec, int N, int force_R, int force_block, in
     c->cur = c->stream;
     const size_t ne = half_elems(c, N);
     for (int k = 0; k < 8; ++k) CK(launch_fill(prec, c->lo[k], ne, 77u + k, c->stream));
+    struct Shape {
+        int R, B, pf;
+        float ms[3];  // per class, the fastest time seen
+    };
+    std::vector<Shape> shapes;
+    const int which_of[3] = {1, 4, 2};  // the hop time_hops times for each class
+    const int Rs[3] = {1, 2, 4}, Bs[3] = {64, 128, 256};
+    for (int pf = 0; pf < (prec == P_F64 ? 1 : 13); ++pf)
+        for (int ri = 0; ri < 3; ++ri)
+            for (int bi = 0; bi < 3; ++bi)
+                if ((force_pf < 0 || pf == force_pf) && (!force_R || Rs[ri] == force_R) &&
+                    (!force_block || Bs[bi] == force_block) && shape_ok(prec, N, Rs[ri], Bs[bi], bi, pf))
+                    shapes.push_back({Rs[ri], Bs[bi], pf, {1e30f, 1e30f, 1e30f}});
     float best[3] = {1e30f, 1e30f, 1e30f}, best0[3] = {1e30f, 1e30f, 1e30f};  // per class: all kinds; kind 0
     int bR[3], bB[3], bP[3], b0R[3], b0B[3];
-    const int which_of[3] = {1, 4, 2};  // the hop time_hops times for each class
     for (int m = 0; m < 3; ++m) {
         bR[m] = b0R[m] = c->hop_R[prec][l][m];
         bB[m] = b0B[m] = c->hop_block[prec][l][m];
         bP[m] = c->hop_kind[prec][l][m];
     }
-    const int Rs[3] = {1, 2, 4}, Bs[3] = {64, 128, 256};
-    // Two sweeps over the shapes, keeping each shape's faster time, so that a
-    // shape timed while the GPU was still ramping its clocks or finishing other
-    // work gets a second chance.
-    for (int sweep = 0; sweep < 2; ++sweep)
-    for (int pf = 0; pf < (prec == P_F64 ? 1 : 12); ++pf) {
-        if (force_pf >= 0 && pf != force_pf) continue;
-        for (int ri = 0; ri < 3; ++ri) {
-            const int R = Rs[ri];
-            if (force_R && R != force_R) continue;
-            for (int bi = 0; bi < 3; ++bi) {
-                const int B = Bs[bi];
-                if (force_block && B != force_block) continue;
-                if (!shape_ok(prec, N, R, B, bi, pf)) continue;
-                for (int m = 0; m < 3; ++m) {
-                    c->hop_R[prec][l][m] = R;
-                    c->hop_block[prec][l][m] = B;
-                    c->hop_kind[prec][l][m] = pf;
+    // A first pass of one launch per shape (after a warm-up launch) finds the contenders;
+    // those within a fifth of the best are timed twice more, five launches each, so that a
+    // shape timed while the GPU was still ramping its clocks or finishing other work gets
+    // another chance.  (Five launches of every shape twice cost 0.8 s on 16^3 x 32 at width
+    // 32, six times a solve of 32 sources; this costs 0.1 s.)
+    for (int sweep = 0; sweep < 3; ++sweep) {
+        float lead[3];
+        for (int m = 0; m < 3; ++m) lead[m] = best[m];
+        for (Shape &s : shapes)
+            for (int m = 0; m < 3; ++m) {
+                if (sweep > 0 && s.ms[m] > 1.2f * lead[m] && !(s.pf == 0 && s.ms[m] <= best0[m])) continue;
+                c->hop_R[prec][l][m] = s.R;
+                c->hop_block[prec][l][m] = s.B;
+                c->hop_kind[prec][l][m] = s.pf;
+                float ms = 0.f;
+                TRY(time_hops(c, prec, N, sweep ? 5 : 1, &ms, which_of[m]));
+                if (!(ms > 0.f)) continue;
+                s.ms[m] = std::min(s.ms[m], ms);
+                if (ms < best[m]) {
+                    best[m] = ms;
+                    bR[m] = s.R;
+                    bB[m] = s.B;
+                    bP[m] = s.pf;
                 }
-                for (int m = 0; m < 3; ++m) {
-                    float ms = 0.f;
-                    TRY(time_hops(c, prec, N, 5, &ms, which_of[m]));
-                    if (ms > 0.f && ms < best[m]) {
-                        best[m] = ms;
-                        bR[m] = R;
-                        bB[m] = B;
-                        bP[m] = pf;
-                    }
-                    if (pf == 0 && ms > 0.f && ms < best0[m]) {
-                        best0[m] = ms;
-                        b0R[m] = R;
-                        b0B[m] = B;
-                    }
+                if (s.pf == 0 && ms < best0[m]) {
+                    best0[m] = ms;
+                    b0R[m] = s.R;
+                    b0B[m] = s.B;
                 }
             }
-        }
     }
     // Another kind replaces the direct kernel only when it is faster by more than
     // 2%: closer than that, which one wins is timing noise (on GB300 the
@@ -604,7 +612,7 @@ extern "C" int dl_set_hop_shape(dl_ctx *c, int precision, int n_rhs, int cls, in
         return fail(DL_EINVAL, "bad arguments");
     const int N = pow2_at_least(n_rhs), l = ilog2(N), ip = inner_prec(c, precision, N), m = cls;
     const int bi = block == 64 ? 0 : (block == 128 ? 1 : (block == 256 ? 2 : -1));
-    if ((R != 1 && R != 2 && R != 4) || bi < 0 || !shape_ok(ip, N, R, block, bi, kind))
+    if ((R != 1 && R != 2 && R != 4) || bi < 0 || kind > 11 || !shape_ok(ip, N, R, block, bi, kind))
         return fail(DL_EINVAL, "launch shape not available for this precision, width and layout");
     c->hop_R[ip][l][m] = R;
     c->hop_block[ip][l][m] = block;
@@ -1295,6 +1303,22 @@ static int tune_for(dl_ctx *c, const SolveCfg &P, int N) {
     return P.prec == P_F64 ? DL_OK : maybe_tune(c, P.prec, N);  // (the FP64 hop has one shape)
 }
 
+// Layout width of a batch of n right-hand sides in a solve of width N.  A last batch
+// of half the width or less takes a narrower layout: the columns without a right-hand
+// side load and store nothing, but their hops cost the full width's instructions (32 + 16
+// sources on 16^3 x 32: 211 ms with both batches in layouts of 32, 187 ms with the
+// second in one of 16).  A
+// resident solve spends nothing on them, a pinned width and a fixed number of
+// iterations (whose result must be the same map in every batch) keep N.
+static int batch_width(dl_ctx *c, const SolveCfg &P, int n, int N) {
+    const int W = pow2_at_least(n), prec = inner_prec(c, P.prec, N);
+    int C = 0;
+    if (W >= N || P.fixed_iters > 0 || c->hop_pinned[prec][ilog2(N)] || inner_prec(c, P.prec, W) != prec ||
+        resident_plan(c, P, N, &C))
+        return N;
+    return W;
+}
+
 static int ensure_resident(dl_ctx *c, int prec) {
     if (c->reslinks_ok[prec]) return DL_OK;
     if (!c->d_reslinks[prec] &&
@@ -1478,10 +1502,12 @@ static int solve_impl(dl_ctx *c, const void *b, void *x, int n_rhs, const dl_sol
     std::vector<OuterState> os;
     for (int j0 = 0; j0 < n_rhs; j0 += N) {
         const int n = std::min(N, n_rhs - j0);
+        const int W = batch_width(c, P, n, N);
+        if (W != N) TRY(tune_for(c, P, W));
         c->cur = c->stream;
-        TRY(canon_to_eo(c, (const double *)b + (size_t)j0 * field, c->b64, n, N, g5, 0, (int)c->Vh));
-        TRY(solve_batch(c, n, N, P, os));
-        TRY(eo_to_canon(c, c->x64, (double *)x + (size_t)j0 * field, n, N, g5, 0, (int)c->Vh));
+        TRY(canon_to_eo(c, (const double *)b + (size_t)j0 * field, c->b64, n, W, g5, 0, (int)c->Vh));
+        TRY(solve_batch(c, n, W, P, os));
+        TRY(eo_to_canon(c, c->x64, (double *)x + (size_t)j0 * field, n, W, g5, 0, (int)c->Vh));
         for (int j = 0; j < n; ++j) {
             const int s = status_of(os[j], P.tol, P.fixed_iters > 0);
             if (stats) {

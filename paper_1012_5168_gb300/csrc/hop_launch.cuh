@@ -39,6 +39,11 @@ cudaError_t go_hop(const HopArgs &a, Launch &l, int kind) {
                     hop_kernel_clov_cap<S, MODE, RED, ccap, 32><<<l.grid, l.block, l.smem, l.stream>>>(a);
                     return cudaGetLastError();
                 }
+                if (a.N == 16) {
+                    clamp_grid(l, resident_blocks(hop_kernel_clov_cap<S, MODE, RED, ccap, 16>, l.block, l.smem));
+                    hop_kernel_clov_cap<S, MODE, RED, ccap, 16><<<l.grid, l.block, l.smem, l.stream>>>(a);
+                    return cudaGetLastError();
+                }
             }
             clamp_grid(l, resident_blocks(hop_kernel_clov<S, MODE, RED>, l.block, l.smem));
             hop_kernel_clov<S, MODE, RED><<<l.grid, l.block, l.smem, l.stream>>>(a);
@@ -53,9 +58,10 @@ cudaError_t go_hop(const HopArgs &a, Launch &l, int kind) {
     }();
     if (kind == 0) {
         if constexpr (cap > 0) {
-            if (a.N == 32) {  // the benchmark width: offsets as compile-time constants
-                clamp_grid(l, resident_blocks(hop_kernel_cap<S, R, MODE, RED, cap, 32>, l.block, l.smem));
-                hop_kernel_cap<S, R, MODE, RED, cap, 32><<<l.grid, l.block, l.smem, l.stream>>>(a);
+            if (a.N == 32 || a.N == 16) {  // the usual widths: offsets as compile-time constants
+                auto k = a.N == 32 ? hop_kernel_cap<S, R, MODE, RED, cap, 32> : hop_kernel_cap<S, R, MODE, RED, cap, 16>;
+                clamp_grid(l, resident_blocks(k, l.block, l.smem));
+                k<<<l.grid, l.block, l.smem, l.stream>>>(a);
                 return cudaGetLastError();
             }
         }
@@ -66,7 +72,9 @@ cudaError_t go_hop(const HopArgs &a, Launch &l, int kind) {
     if (kind == 10) {  // the direct FP32 kernel under a wider register cap (80 plain, 96 fused)
         if constexpr (std::is_same<S, float>::value && R == 1) {
             constexpr int wcap = MODE == MODE_PLAIN ? 80 : 96;
-            auto k = a.N == 32 ? hop_kernel_cap<S, 1, MODE, RED, wcap, 32> : hop_kernel_cap<S, 1, MODE, RED, wcap>;
+            auto k = a.N == 32   ? hop_kernel_cap<S, 1, MODE, RED, wcap, 32>
+                     : a.N == 16 ? hop_kernel_cap<S, 1, MODE, RED, wcap, 16>
+                                 : hop_kernel_cap<S, 1, MODE, RED, wcap>;
             clamp_grid(l, resident_blocks(k, l.block, l.smem));
             k<<<l.grid, l.block, l.smem, l.stream>>>(a);
             return cudaGetLastError();
@@ -123,6 +131,23 @@ cudaError_t go_hop(const HopArgs &a, Launch &l, int kind) {
         l.grid = (l.num_sms > 0 ? l.num_sms : 1) * (res < 16 ? res : 16);
         kern<<<l.grid, l.block, l.smem, l.stream>>>(a);
         return cudaGetLastError();
+    }
+    if (kind == 12) {  // warp-staged at width 16, two sites per warp (FP32), two stages
+        if constexpr (std::is_same<S, float>::value && R == 1) {
+            if (a.N != 16) return cudaErrorInvalidValue;
+            static size_t opted = 0;
+            static std::mutex m;
+            auto kern = hop_kernel_ws<S, 1, MODE, RED, 2, 2>;
+            l.block = WS_WARPS * 32;
+            l.smem = WsShape<S, 1, 2, 2>::WB * WS_WARPS;
+            const cudaError_t e = opt_in_smem(kern, l.smem, opted, m);
+            if (e != cudaSuccess) return e;
+            const int res = resident_blocks(kern, l.block, l.smem);
+            l.grid = (l.num_sms > 0 ? l.num_sms : 1) * (res < 16 ? res : 16);
+            kern<<<l.grid, l.block, l.smem, l.stream>>>(a);
+            return cudaGetLastError();
+        }
+        return cudaErrorInvalidValue;
     }
     if (kind == 6) {  // direct loads, packed FP32 arithmetic (FP32 storage, R = 1)
         if constexpr (std::is_same<S, float>::value && R == 1) {

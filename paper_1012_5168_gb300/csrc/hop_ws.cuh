@@ -18,6 +18,9 @@
 // (the next site's links land while the current site still uses its own) and
 // the NST mbarriers.
 //
+// Width 16 (FP32, kernel kind 12): a warp owns two consecutive sites, one per half
+// warp (SPW = 2); a stage holds the two neighbour blocks, a link row both sites'.
+//
 // Every wait is bounded: when one runs out, the warp records A.err[0], stops,
 // waits (bounded again) for the copies it has issued, and leaves the site
 // loop; if a drain wait runs out as well it records A.err[1] (copies may then
@@ -35,10 +38,10 @@ constexpr int WS_WARPS = 4;  // warps per block of the warp-staged hop
 // NSTO = 2 (kernel kind 11) keeps one copy in flight and so fits about twice
 // the warps per SM: on GB300 that runs the fused hops faster (their epilogue
 // loads gain from the extra warps) and the plain hop slower.
-template <typename S, int R, int NSTO = 0>
+template <typename S, int R, int NSTO = 0, int SPW = 1>
 struct WsShape {
-    static constexpr uint32_t SB = 12u * 32u * R * cbytes<S>();  // one neighbour block [12][N]
-    static constexpr uint32_t LB = 8u * 9u * cbytes<S>();        // one site's eight links
+    static constexpr uint32_t SB = 12u * 32u * R * cbytes<S>();  // SPW neighbour blocks [12][N], N = 32 R / SPW
+    static constexpr uint32_t LB = SPW * 8u * 9u * cbytes<S>();  // SPW sites' eight links
     static constexpr int NST = NSTO ? NSTO : (SB <= 1536 ? 6 : (SB <= 3072 ? 4 : 3));
     static constexpr size_t WB = 64 + (size_t)NST * SB + 2 * (size_t)LB;  // bytes per warp
 };
@@ -61,11 +64,11 @@ __device__ __forceinline__ int nbr_of_dir(const Site &s, const Geom &g, int d) {
     return i >> 1;
 }
 
-template <typename S, int R, int MODE, int RED, int NSTO = 0>
+template <typename S, int R, int MODE, int RED, int NSTO = 0, int SPW = 1>
 __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
     typedef typename Real<S>::type T;
-    typedef WsShape<S, R, NSTO> W;
-    constexpr int N = 32 * R;
+    typedef WsShape<S, R, NSTO, SPW> W;
+    constexpr int N = 32 * R / SPW, LPS = 32 / SPW;  // right-hand sides; lanes per site
     constexpr int NST = W::NST;
     constexpr int NV = RedCount<RED>::n > 0 ? RedCount<RED>::n : 1;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -77,10 +80,11 @@ __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
 
     const int gw = blockIdx.x * WS_WARPS + warp;
     const int tw = gridDim.x * WS_WARPS;
-    const int nsite = A.cb_end - A.cb_begin;
+    const int nsite = (A.cb_end - A.cb_begin) / SPW;  // (the number of even sites is a multiple of 8)
     const int nmy = gw < nsite ? (nsite - 1 - gw) / tw + 1 : 0;
     const int nsteps = nmy * 8;
-    const int r0 = lane * R;
+    const int sub = SPW > 1 ? lane / LPS : 0;  // which of the warp's sites
+    const int r0 = (SPW > 1 ? lane % LPS : lane) * R;
     const T cD = from_double<T>(A.c);
     const S *in = reinterpret_cast<const S *>(A.in);
     const S *g8 = reinterpret_cast<const S *>(A.gauge8);
@@ -91,21 +95,26 @@ __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
     }
     __syncwarp();
 
-    // Lane d < 8 holds the neighbour of direction d of the site being issued.
+    // Lane 8 s + d holds the neighbour of direction d of the s-th site being issued.
     int nb_issue = 0;
     auto issue = [&](int k) {
         const int j = k >> 3, d = k & 7, slot = k % NST;
-        const int cb = A.cb_begin + gw + j * tw;
+        const int cb = A.cb_begin + (gw + j * tw) * SPW;
         if (d == 0) {
-            const Site st = decode(__ldg(A.coords + (size_t)A.p * A.g.Vh + cb), A.g);
-            nb_issue = lane < 8 ? nbr_of_dir(st, A.g, lane) : 0;
+            const Site st = decode(__ldg(A.coords + (size_t)A.p * A.g.Vh + cb + (lane < 8 * SPW ? lane / 8 : 0)), A.g);
+            nb_issue = lane < 8 * SPW ? nbr_of_dir(st, A.g, lane & 7) : 0;
         }
-        const int nb = __shfl_sync(0xffffffffu, nb_issue, d);
+        int nb[SPW];
+#pragma unroll
+        for (int q = 0; q < SPW; ++q) nb[q] = __shfl_sync(0xffffffffu, nb_issue, d + 8 * q);
         fence_proxy_async();  // this warp's reads of the slot come before the async writes into it
         __syncwarp();
         if (lane == 0) {
             mbar_expect_tx(full + slot, W::SB + (d == 0 ? W::LB : 0u));
-            bulk_copy(stg + (size_t)slot * W::SB, in + (size_t)nb * 12 * N * 2, W::SB, full + slot);
+#pragma unroll
+            for (int q = 0; q < SPW; ++q)
+                bulk_copy(stg + (size_t)slot * W::SB + q * (W::SB / SPW), in + (size_t)nb[q] * 12 * N * 2, W::SB / SPW,
+                          full + slot);
             if (d == 0)
                 bulk_copy(lnk + (size_t)(j & 1) * W::LB, g8 + ((size_t)A.p * A.g.Vh + cb) * 8 * 18, W::LB,
                           full + slot);
@@ -123,9 +132,9 @@ __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
     bool ok = true;
     int k = 0;  // next step to wait for
     for (int j = 0; j < nmy && ok; ++j) {
-        const int cb = A.cb_begin + gw + j * tw;
+        const int cb = A.cb_begin + (gw + j * tw) * SPW + sub;
         // (the link rows carry the time boundary factor)
-        const unsigned char *lrow = lnk + (size_t)(j & 1) * W::LB;
+        const unsigned char *lrow = lnk + (size_t)(j & 1) * W::LB + sub * (W::LB / SPW);
         cx<T> acc[R][12];
 #pragma unroll
         for (int r = 0; r < R; ++r)
@@ -136,7 +145,7 @@ __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
             const int slot = k % NST;                                                                  \
             ok = __all_sync(0xffffffffu, mbar_wait(full + slot, (uint32_t)((k / NST) & 1)));           \
             if (ok) {                                                                                  \
-                tma_compute<S, R, D>(stg + (size_t)slot * W::SB, lrow, N, r0,                          \
+                tma_compute<S, R, D>(stg + (size_t)slot * W::SB + sub * (W::SB / SPW), lrow, N, r0,    \
                                      false, acc);            \
                 __syncwarp();                                                                          \
                 if (k + NST < nsteps) {                                                                \
@@ -214,7 +223,7 @@ __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
         // reduction reuses the staging memory from byte 64 on (WS_WARPS * 32 * R *
         // NV complex, at most 10 kB, below the WS_WARPS * WB bytes of the block).
         __syncthreads();
-        block_reduce<R, NV, T>(red, 32, N, A.partials, smem + 64);
+        block_reduce<R, NV, T>(red, LPS, N, A.partials, smem + 64);
     }
 }
 
