@@ -1432,8 +1432,8 @@ static int solve_batch(dl_ctx *c, int n, int N, const SolveCfg &P, std::vector<O
             ResArgs a;
             for (int k = 0; k < 8; ++k) a.f[k] = c->lo[k];
             a.links = c->d_reslinks[prec];
-            a.coords = c->d_coords;
             a.g = c->g;
+            for (int mu = 0; mu < 3; ++mu) a.div[mu] = (uint32_t)((1ull << 32) / (uint64_t)c->dims[mu]) + 1;
             a.N = N;
             a.k2 = k2;
             a.st = c->d_rhs;

@@ -22,7 +22,10 @@
 // share 32 sites, warp q taking direction mu = q forward and backward: all 33
 // loads of a thread are in flight at once, the four partial sums meet in shared
 // memory, and warp q goes on with spin q (three of the twelve components) in
-// the epilogue and in the vector updates (3400 cycles).
+// the epilogue and in the vector updates (3400 cycles).  The vector updates load two
+// sites a step, and the coordinates are computed (every cluster barrier empties L1 of a
+// table of them): CGNR on 8^3 x 16 from 11.0 to 10.2 ms a solve (12.2 ms step by step), 24
+// right-hand sides of a fermion force there from 24.5 to 22.3 ms (30.0 ms).
 //
 // Layout.  The inner fields belong to this kernel alone: per right-hand side
 // [tile of 32 sites][12][32] complex.  A warp reads 256 contiguous bytes per
@@ -50,7 +53,6 @@ constexpr int RES_THREADS = 512;               // one block per SM, 128 register
 constexpr int RES_GROUPS = RES_THREADS / 128;  // groups of four warps, 32 sites each
 constexpr int RES_ROUND = 32 * RES_GROUPS;     // sites of a block in flight
 constexpr int RES_MAX_C = 16;                  // blocks per cluster
-constexpr int RES_COORDS = 512;                // sites per parity whose coordinates a block keeps in shared memory
 
 // Complex values of one right-hand side's inner field, and of the links of both parities.
 inline size_t res_field_elems(long Vh) { return (size_t)((Vh + 31) / 32) * 384; }
@@ -59,8 +61,8 @@ inline size_t res_link_elems(long Vh) { return (size_t)2 * ((Vh + 31) / 32) * 32
 struct ResArgs {
     void *f[8];             // x r rhat p v s t tmp: [rhs][tile][12][32] complex of S
     const void *links;      // [2][tile][36][32] pairs of complex of S
-    const uint32_t *coords;
     Geom g;
+    uint32_t div[3];        // floor(2^32 / d) + 1 for d = L_x, L_y, L_z
     int N;                  // width of the FP64 fields
     double k2;              // kappa^2
     RhsState *st;
@@ -98,7 +100,6 @@ struct ResShared {
     RhsState rhs;
     cx<T> alpha, omega, beta;                        // the scalars in arithmetic precision
     int active, next;
-    uint32_t coords[2][RES_COORDS];
 };
 // A conversion from FP64 costs about as much as an FP64 instruction: one thread
 // makes them for all.
@@ -109,6 +110,21 @@ template <typename T> __device__ __forceinline__ void res_publish(ResShared<T> &
     sh.beta = mk((T)s.beta.x, (T)s.beta.y);
     sh.active = s.active;
     sh.next = s.next_active;
+}
+
+// Coordinates of checkerboard site cb of parity par: quotients n / d by multiplication, exact
+// for n d < 2^32 and d > 1 (n is below 2^15 here, an extent at most 256).  A table of them would be one more load
+// round trip, since every cluster barrier empties L1.
+__device__ __forceinline__ Site res_site(int cb, int par, const Geom &g, const uint32_t (&div)[3]) {
+    Site s;
+    const int row = (int)__umulhi(2 * (uint32_t)cb, div[0]), zt = (int)__umulhi((uint32_t)row, div[1]);
+    const int t = (int)__umulhi((uint32_t)zt, div[2]);
+    s.c[1] = row - zt * g.L[1];
+    s.c[2] = zt - t * g.L[2];
+    s.c[3] = t;
+    s.c[0] = 2 * (cb - row * (g.L[0] >> 1)) + ((s.c[1] + s.c[2] + t + par) & 1);
+    s.i = 2 * cb + (s.c[0] & 1);
+    return s;
 }
 
 // Barrier of the four warps of a group.
@@ -190,12 +206,23 @@ __device__ __forceinline__ void res_mu(const S *in, const S *lk, const Geom &g, 
     const uint32_t tf = res_tile(nbr_fwd(st, g, MU)), tb = res_tile(nbr_bwd(st, g, MU));
     load_project<S, 1, MU, -1, false>(in + 2 * (size_t)tf, 32, hf);
     load_project<S, 1, MU, +1, false>(in + 2 * (size_t)tb, 32, hb);
-#pragma unroll
-    for (int c = 0; c < 12; ++c) acc[c] = zero<T>();
+    // w+ = U h+ and w- = V^dag h-: the pair contributes [w+ + w-; X^dag (w- - w+)], X being the
+    // projection's map (no sums with zeros, and one permutation for both)
     su3_mul<T, false>(u, hf[0], w);
-    reconstruct<T, MU, -1>(w, acc);
-    su3_mul<T, true>(v, hb[0], w);
-    reconstruct<T, MU, +1>(w, acc);
+    {
+        cx<T> y[6];
+        su3_mul<T, true>(v, hb[0], y);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            acc[k] = w[k] + y[k];
+            w[k] = y[k] - w[k];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        acc[6 + k] = MU == 0 ? tmi(w[3 + k]) : MU == 1 ? w[3 + k] : MU == 2 ? tmi(w[k]) : w[k];
+        acc[9 + k] = MU == 0 ? tmi(w[k]) : MU == 1 ? -w[k] : MU == 2 ? ti(w[3 + k]) : w[3 + k];
+    }
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
@@ -226,7 +253,6 @@ __global__ void __launch_bounds__(RES_THREADS, 1) resident_kernel(ResArgs A) {
     const int first = grp * 32 + lane;  // this thread's first site; the next ones are RES_ROUND apart
     const int c3 = 3 * q;               // its components c3 .. c3 + 2 (spin q)
 
-    const bool local = c1 - c0 <= RES_COORDS;
     auto fence = [&] {
         if (C == 1) __syncthreads();
         else cluster.sync();
@@ -237,7 +263,7 @@ __global__ void __launch_bounds__(RES_THREADS, 1) resident_kernel(ResArgs A) {
         const int cb = c0 + i;
         cx<T>(*part)[32] = sh.part[grp][q];
         if (i < n) {
-            const Site st = decode(local ? sh.coords[par][cb - c0] : __ldg(A.coords + (size_t)par * Vh + cb), A.g);
+            const Site st = res_site(cb, par, A.g, A.div);
             const S *lk = (const S *)A.links +
                           ((size_t)(par * ((Vh + 31) >> 5) + (cb >> 5)) * 36 * 32 + (cb & 31)) * 4;
             if (q == 0) res_mu<S, 0>(in, lk, A.g, st, d, part, lane);
@@ -254,13 +280,6 @@ __global__ void __launch_bounds__(RES_THREADS, 1) resident_kernel(ResArgs A) {
         }
         res_bar(grp);
     };
-
-    // the coordinates of this block's sites: every cluster barrier empties L1 of them
-    if (local)
-        for (int k = tid; k < 2 * (c1 - c0); k += RES_THREADS) {
-            const int par = k >= c1 - c0;
-            sh.coords[par][k - par * (c1 - c0)] = A.coords[(size_t)par * Vh + c0 + k - par * (c1 - c0)];
-        }
 
     // ---- phase set-up: fields from the FP64 residual
     const OuterState &o = A.os[rg];
@@ -387,27 +406,37 @@ __global__ void __launch_bounds__(RES_THREADS, 1) resident_kernel(ResArgs A) {
             __syncthreads();
             n = sh.active ? nit : 0;  // after a breakdown nothing more is touched
             al = sh.alpha;
-            for (int i = first; i < n; i += RES_ROUND) {
-                const uint32_t t = res_tile(c0 + i);
-                cx<T> rv[3], vv[3], xv[3], pv[3];
+            for (int i0 = first; i0 < n; i0 += 2 * RES_ROUND) {  // two sites' loads in flight
+                cx<T> rv[2][3], vv[2][3], xv[2][3], pv[2][3];
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    rv[a] = res_ld<S>(R, t, c3 + a);
-                    vv[a] = res_ld<S>(V, t, c3 + a);
-                    if (CG) {
-                        xv[a] = res_ld<S>(X, t, c3 + a);
-                        pv[a] = res_ld<S>(P, t, c3 + a);
+                for (int h = 0; h < 2; ++h) {
+                    const int i = i0 + h * RES_ROUND;
+                    const uint32_t t = res_tile(c0 + (i < n ? i : i0));
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        rv[h][a] = res_ld<S>(R, t, c3 + a);
+                        vv[h][a] = res_ld<S>(V, t, c3 + a);
+                        if (CG) {
+                            xv[h][a] = res_ld<S>(X, t, c3 + a);
+                            pv[h][a] = res_ld<S>(P, t, c3 + a);
+                        }
                     }
                 }
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    if (CG) {
-                        res_st<S>(X, t, c3 + a, xv[a] + al.re * pv[a]);
-                        const cx<T> z = res_round<S>(rv[a] - (q >= 2 ? -al.re : al.re) * vv[a]);
-                        res_st<S>(R, t, c3 + a, z);
-                        cjmac(red[0], z, z);
-                    } else {
-                        res_st<S>(SS, t, c3 + a, rv[a] - al * vv[a]);
+                for (int h = 0; h < 2; ++h) {
+                    const int i = i0 + h * RES_ROUND;
+                    if (i >= n) break;
+                    const uint32_t t = res_tile(c0 + i);
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        if (CG) {
+                            res_st<S>(X, t, c3 + a, xv[h][a] + al.re * pv[h][a]);
+                            const cx<T> z = res_round<S>(rv[h][a] - (q >= 2 ? -al.re : al.re) * vv[h][a]);
+                            res_st<S>(R, t, c3 + a, z);
+                            cjmac(red[0], z, z);
+                        } else {
+                            res_st<S>(SS, t, c3 + a, rv[h][a] - al * vv[h][a]);
+                        }
                     }
                 }
             }
@@ -427,28 +456,39 @@ __global__ void __launch_bounds__(RES_THREADS, 1) resident_kernel(ResArgs A) {
         }
         __syncthreads();
         const cx<T> om = sh.omega, be = sh.beta;
-        for (int i = first; i < (sh.active ? nit : 0); i += RES_ROUND) {
-            const uint32_t t = res_tile(c0 + i);
-            cx<T> xv[3], pv[3], sv[3], tv[3], vv[3];
+        n = sh.active ? nit : 0;
+        for (int i0 = first; i0 < n; i0 += 2 * RES_ROUND) {
+            cx<T> xv[2][3], pv[2][3], sv[2][3], tv[2][3], vv[2][3];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                pv[a] = res_ld<S>(P, t, c3 + a);
-                tv[a] = res_ld<S>(TT, t, c3 + a);
-                if (!CG) {
-                    xv[a] = res_ld<S>(X, t, c3 + a);
-                    sv[a] = res_ld<S>(SS, t, c3 + a);
-                    vv[a] = res_ld<S>(V, t, c3 + a);
+            for (int h = 0; h < 2; ++h) {
+                const int i = i0 + h * RES_ROUND;
+                const uint32_t t = res_tile(c0 + (i < n ? i : i0));
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    pv[h][a] = res_ld<S>(P, t, c3 + a);
+                    tv[h][a] = res_ld<S>(TT, t, c3 + a);
+                    if (!CG) {
+                        xv[h][a] = res_ld<S>(X, t, c3 + a);
+                        sv[h][a] = res_ld<S>(SS, t, c3 + a);
+                        vv[h][a] = res_ld<S>(V, t, c3 + a);
+                    }
                 }
             }
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                if (CG) {
-                    res_st<S>(P, t, c3 + a, (q >= 2 ? (T)-1 : (T)1) * tv[a] + be.re * pv[a]);
-                } else {
-                    res_st<S>(X, t, c3 + a, xv[a] + al * pv[a] + om * sv[a]);
-                    const cx<T> rn = sv[a] - om * tv[a];
-                    res_st<S>(R, t, c3 + a, rn);
-                    res_st<S>(P, t, c3 + a, rn + be * (pv[a] - om * vv[a]));
+            for (int h = 0; h < 2; ++h) {
+                const int i = i0 + h * RES_ROUND;
+                if (i >= n) break;
+                const uint32_t t = res_tile(c0 + i);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    if (CG) {
+                        res_st<S>(P, t, c3 + a, (q >= 2 ? (T)-1 : (T)1) * tv[h][a] + be.re * pv[h][a]);
+                    } else {
+                        res_st<S>(X, t, c3 + a, xv[h][a] + al * pv[h][a] + om * sv[h][a]);
+                        const cx<T> rn = sv[h][a] - om * tv[h][a];
+                        res_st<S>(R, t, c3 + a, rn);
+                        res_st<S>(P, t, c3 + a, rn + be * (pv[h][a] - om * vv[h][a]));
+                    }
                 }
             }
         }

@@ -22,7 +22,8 @@ torch = pytest.importorskip("torch")
 
 @pytest.mark.parametrize("dims, n, batch", [((2, 2, 2, 2), 3, 4), ((4, 4, 4, 4), 64, 64), ((6, 2, 4, 6), 1, 1),
                                             ((6, 6, 6, 8), 5, 32), ((6, 10, 4, 12), 7, 4), ((8, 8, 8, 16), 1, 1),
-                                            ((4, 6, 2, 4), 35, 32)])
+                                            ((4, 6, 2, 4), 35, 32), ((256, 2, 2, 2), 2, 2),
+                                            ((2, 256, 2, 4), 1, 1)])
 @pytest.mark.parametrize("prec, method", [(1, 0), (2, 0), (1, 1)])
 def test_resident_solve(lib, dims, n, batch, prec, method):
     kappa, tol = 0.11, 1e-11
