@@ -247,7 +247,7 @@ static int hop_class(int mode, int red) {
 }
 
 // clov: the clover solve's inner hop A^-1 D (A^-1 of the output parity p in the epilogue;
-// FP64, FP32 or BF16 storage, the direct kernel with one right-hand side per thread).
+// FP64, FP32 or BF16 storage; go_hop's own rule picks the kernel, one right-hand side per thread).
 static int do_hop(dl_ctx *c, int prec, int mode, int red, void *out, const void *in, const void *y, const void *z,
                   const void *rhat, int p, int N, double coef, int cb0, int cb1, double2 *partials, int *nblocks,
                   int ffmt = 0, const RhsState *act = nullptr, bool clov = false) {

@@ -44,4 +44,25 @@ __device__ __forceinline__ void clover_inv_apply(const S *m, cx<T> (&acc)[12]) {
     }
 }
 
+// The same from shared memory (FP32, 16-byte aligned): two elements per load.
+__device__ __forceinline__ void clover_inv_apply_smem(const float4 *m, cx<float> (&acc)[12]) {
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+        cx<float> v[6];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) v[j] = acc[6 * b + j];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            cx<float> o = zero<float>();
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const float4 t = m[b * 18 + i * 3 + j];
+                cmac(o, mk(t.x, t.y), v[2 * j]);
+                cmac(o, mk(t.z, t.w), v[2 * j + 1]);
+            }
+            acc[6 * b + i] = o;
+        }
+    }
+}
+
 }  // namespace dl

@@ -511,16 +511,11 @@ __global__ void __maxnreg__(CAP) hop_kernel_cap(HopArgs A) {
 }
 
 // Clover direct kernel (one right-hand side per thread): the inner hops of the
-// clover operator's asymmetric Schur system, A^-1 D.
+// clover operator's asymmetric Schur system, A^-1 D (FP64, BF16, and FP32 at widths
+// other than 32 and 16, which go warp by warp: hop_ws.cuh).
 template <typename S, int MODE, int RED>
 __global__ void __launch_bounds__(256) hop_kernel_clov(HopArgs A) {
     hop_body<S, 1, MODE, RED, 0, 0, 1>(A);
-}
-// The same under the direct FP32 kernels' register caps, with the width a
-// compile-time constant.
-template <typename S, int MODE, int RED, int CAP, int NC>
-__global__ void __maxnreg__(CAP) hop_kernel_clov_cap(HopArgs A) {
-    hop_body<S, 1, MODE, RED, NC, 0, 1>(A);
 }
 
 // Packed-arithmetic direct kernel (FP32 storage, one right-hand side per thread).

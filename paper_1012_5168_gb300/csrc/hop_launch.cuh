@@ -28,22 +28,32 @@ inline cudaError_t opt_in_smem(K kernel, size_t smem, size_t &opted, std::mutex 
     return e;
 }
 
+// Warp-staged clover hop (FP32, two stages, SPW sites of 32 / SPW right-hand sides per warp).
+template <int SPW, int MODE, int RED>
+cudaError_t go_clov_ws(const HopArgs &a, Launch &l) {
+    static size_t opted = 0;
+    static std::mutex m;
+    auto kern = hop_kernel_ws<float, 1, MODE, RED, 2, SPW, true>;
+    l.block = WS_WARPS * 32;
+    l.smem = WsShape<float, 1, 2, SPW, true>::WB * WS_WARPS;
+    const cudaError_t e = opt_in_smem(kern, l.smem, opted, m);
+    if (e != cudaSuccess) return e;
+    const int res = resident_blocks(kern, l.block, l.smem);
+    l.grid = (l.num_sms > 0 ? l.num_sms : 1) * (res < 16 ? res : 16);
+    kern<<<l.grid, l.block, l.smem, l.stream>>>(a);
+    return cudaGetLastError();
+}
+
 template <typename S, int R, int MODE, int RED>
 cudaError_t go_hop(const HopArgs &a, Launch &l, int kind) {
-    if (a.clovinv) {  // clover: the direct kernel with A^-1 in the epilogue, one right-hand side per thread
+    if (a.clovinv) {  // clover: A^-1 in the epilogue, one right-hand side per thread
         if constexpr (R == 1) {
-            constexpr int ccap = HopRegCap<S, 1, MODE, RED>::n;
-            if constexpr (ccap > 0) {
-                if (a.N == 32) {
-                    clamp_grid(l, resident_blocks(hop_kernel_clov_cap<S, MODE, RED, ccap, 32>, l.block, l.smem));
-                    hop_kernel_clov_cap<S, MODE, RED, ccap, 32><<<l.grid, l.block, l.smem, l.stream>>>(a);
-                    return cudaGetLastError();
-                }
-                if (a.N == 16) {
-                    clamp_grid(l, resident_blocks(hop_kernel_clov_cap<S, MODE, RED, ccap, 16>, l.block, l.smem));
-                    hop_kernel_clov_cap<S, MODE, RED, ccap, 16><<<l.grid, l.block, l.smem, l.stream>>>(a);
-                    return cudaGetLastError();
-                }
+            // FP32, widths 32 and 16: warp-staged, A^-1 copied in with the links.  16^3 x 32,
+            // width 32: 136 us plain, 158 and 173 fused, where the direct kernel with its
+            // 1152 bytes of links and A^-1 per thread took 147, 203 and 216.
+            if constexpr (std::is_same<S, float>::value) {
+                if (a.N == 32) return go_clov_ws<1, MODE, RED>(a, l);
+                if (a.N == 16) return go_clov_ws<2, MODE, RED>(a, l);
             }
             clamp_grid(l, resident_blocks(hop_kernel_clov<S, MODE, RED>, l.block, l.smem));
             hop_kernel_clov<S, MODE, RED><<<l.grid, l.block, l.smem, l.stream>>>(a);

@@ -21,6 +21,9 @@
 // Width 16 (FP32, kernel kind 12): a warp owns two consecutive sites, one per half
 // warp (SPW = 2); a stage holds the two neighbour blocks, a link row both sites'.
 //
+// Clover (CLOV): the sites' A^-1 come with their link rows (double-buffered like them)
+// and multiply the result before the epilogue.
+//
 // Every wait is bounded: when one runs out, the warp records A.err[0], stops,
 // waits (bounded again) for the copies it has issued, and leaves the site
 // loop; if a drain wait runs out as well it records A.err[1] (copies may then
@@ -38,12 +41,13 @@ constexpr int WS_WARPS = 4;  // warps per block of the warp-staged hop
 // NSTO = 2 (kernel kind 11) keeps one copy in flight and so fits about twice
 // the warps per SM: on GB300 that runs the fused hops faster (their epilogue
 // loads gain from the extra warps) and the plain hop slower.
-template <typename S, int R, int NSTO = 0, int SPW = 1>
+template <typename S, int R, int NSTO = 0, int SPW = 1, bool CLOV = false>
 struct WsShape {
     static constexpr uint32_t SB = 12u * 32u * R * cbytes<S>();  // SPW neighbour blocks [12][N], N = 32 R / SPW
     static constexpr uint32_t LB = SPW * 8u * 9u * cbytes<S>();  // SPW sites' eight links
+    static constexpr uint32_t CB = CLOV ? SPW * 72u * cbytes<S>() : 0;  // SPW sites' A^-1
     static constexpr int NST = NSTO ? NSTO : (SB <= 1536 ? 6 : (SB <= 3072 ? 4 : 3));
-    static constexpr size_t WB = 64 + (size_t)NST * SB + 2 * (size_t)LB;  // bytes per warp
+    static constexpr size_t WB = 64 + (size_t)NST * SB + 2 * (size_t)(LB + CB);  // bytes per warp
 };
 
 // Checkerboard index of the neighbour in hop direction d (d = 2 mu: x + mu,
@@ -64,10 +68,10 @@ __device__ __forceinline__ int nbr_of_dir(const Site &s, const Geom &g, int d) {
     return i >> 1;
 }
 
-template <typename S, int R, int MODE, int RED, int NSTO = 0, int SPW = 1>
+template <typename S, int R, int MODE, int RED, int NSTO = 0, int SPW = 1, bool CLOV = false>
 __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
     typedef typename Real<S>::type T;
-    typedef WsShape<S, R, NSTO, SPW> W;
+    typedef WsShape<S, R, NSTO, SPW, CLOV> W;
     constexpr int N = 32 * R / SPW, LPS = 32 / SPW;  // right-hand sides; lanes per site
     constexpr int NST = W::NST;
     constexpr int NV = RedCount<RED>::n > 0 ? RedCount<RED>::n : 1;
@@ -77,6 +81,7 @@ __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
     uint64_t *full = reinterpret_cast<uint64_t *>(wbase);
     unsigned char *stg = wbase + 64;
     unsigned char *lnk = stg + (size_t)NST * W::SB;
+    unsigned char *clv = lnk + 2 * (size_t)W::LB;
 
     const int gw = blockIdx.x * WS_WARPS + warp;
     const int tw = gridDim.x * WS_WARPS;
@@ -110,13 +115,17 @@ __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
         fence_proxy_async();  // this warp's reads of the slot come before the async writes into it
         __syncwarp();
         if (lane == 0) {
-            mbar_expect_tx(full + slot, W::SB + (d == 0 ? W::LB : 0u));
+            mbar_expect_tx(full + slot, W::SB + (d == 0 ? W::LB + W::CB : 0u));
 #pragma unroll
             for (int q = 0; q < SPW; ++q)
                 bulk_copy(stg + (size_t)slot * W::SB + q * (W::SB / SPW), in + (size_t)nb[q] * 12 * N * 2, W::SB / SPW,
                           full + slot);
             if (d == 0)
                 bulk_copy(lnk + (size_t)(j & 1) * W::LB, g8 + ((size_t)A.p * A.g.Vh + cb) * 8 * 18, W::LB,
+                          full + slot);
+            if (CLOV && d == 0)
+                bulk_copy(clv + (size_t)(j & 1) * W::CB,
+                          reinterpret_cast<const S *>(A.clovinv) + ((size_t)A.p * A.g.Vh + cb) * 72 * 2, W::CB,
                           full + slot);
         }
     };
@@ -159,6 +168,9 @@ __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
         DL_WS_STEP(4) DL_WS_STEP(5) DL_WS_STEP(6) DL_WS_STEP(7)
 #undef DL_WS_STEP
         if (!ok) break;
+        if constexpr (CLOV)
+            clover_inv_apply_smem(reinterpret_cast<const float4 *>(clv + (size_t)(j & 1) * W::CB + sub * (W::CB / SPW)),
+                                  acc[0]);
         const size_t base = (size_t)cb * 12 * N * 2 + (size_t)r0 * 2;
         S *out = reinterpret_cast<S *>(A.out);
 #pragma unroll
