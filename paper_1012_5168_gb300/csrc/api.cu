@@ -285,6 +285,13 @@ static int do_hop(dl_ctx *c, int prec, int mode, int red, void *out, const void 
                 : prec == P_F64 ? (const void *)c->d_clovinv64
                 : f32           ? (const void *)c->d_clovinv32
                                 : (const void *)c->d_clovinv16;
+    // Evict-first for the streams once a timeslice of the input exceeds 8 MB: the hop reuses
+    // three of them, and a line read from both dies takes its place in both halves of L2.
+    // 24^3 x 48, FP32, width 32 (21 MB): the fused hops from 0.906 and 0.907 to 0.761 and
+    // 0.770 ms; width 16 (10.6 MB): the same within 1%.  16^3 x 32, width 32 (6.3 MB): the
+    // hops alone the same, a solve 0.7% slower with it, since the vector updates find less
+    // of v, s and t in L2.
+    a.stream = (size_t)c->g.V3h * 24 * N * storage_bytes(prec) > ((size_t)8 << 20);
     const int m = hop_class(mode, red);  // the shape tables' entry
     int R = (wide || clov) ? 1 : c->hop_R[prec][ilog2(N)][m];
     if (R > N) R = N;
@@ -510,13 +517,14 @@ static int tune_hop(dl_ctx *c, int prec, int N, int force_R, int force_block, in
                 if ((force_pf < 0 || pf == force_pf) && (!force_R || Rs[ri] == force_R) &&
                     (!force_block || Bs[bi] == force_block) && shape_ok(prec, N, Rs[ri], Bs[bi], bi, pf))
                     shapes.push_back({Rs[ri], Bs[bi], pf, {1e30f, 1e30f, 1e30f}});
-    float best[3] = {1e30f, 1e30f, 1e30f}, best0[3] = {1e30f, 1e30f, 1e30f};  // per class: all kinds; kind 0
-    int bR[3], bB[3], bP[3], b0R[3], b0B[3];
+    float best[3] = {1e30f, 1e30f, 1e30f}, best0[3] = {1e30f, 1e30f, 1e30f};  // per class: all kinds; direct
+    int bR[3], bB[3], bP[3], b0R[3], b0B[3], b0P[3] = {0, 0, 0};
     for (int m = 0; m < 3; ++m) {
         bR[m] = b0R[m] = c->hop_R[prec][l][m];
         bB[m] = b0B[m] = c->hop_block[prec][l][m];
         bP[m] = c->hop_kind[prec][l][m];
     }
+    auto direct = [](int pf) { return pf == 0 || pf == 10; };
     // A first pass of one launch per shape (after a warm-up launch) finds the contenders;
     // those within a fifth of the best are timed twice more, five launches each, so that a
     // shape timed while the GPU was still ramping its clocks or finishing other work gets
@@ -527,7 +535,7 @@ static int tune_hop(dl_ctx *c, int prec, int N, int force_R, int force_block, in
         for (int m = 0; m < 3; ++m) lead[m] = best[m];
         for (Shape &s : shapes)
             for (int m = 0; m < 3; ++m) {
-                if (sweep > 0 && s.ms[m] > 1.2f * lead[m] && !(s.pf == 0 && s.ms[m] <= best0[m])) continue;
+                if (sweep > 0 && s.ms[m] > 1.2f * lead[m] && !(direct(s.pf) && s.ms[m] <= best0[m])) continue;
                 c->hop_R[prec][l][m] = s.R;
                 c->hop_block[prec][l][m] = s.B;
                 c->hop_kind[prec][l][m] = s.pf;
@@ -541,21 +549,23 @@ static int tune_hop(dl_ctx *c, int prec, int N, int force_R, int force_block, in
                     bB[m] = s.B;
                     bP[m] = s.pf;
                 }
-                if (s.pf == 0 && ms < best0[m]) {
+                if (direct(s.pf) && ms < best0[m]) {
                     best0[m] = ms;
+                    b0P[m] = s.pf;
                     b0R[m] = s.R;
                     b0B[m] = s.B;
                 }
             }
     }
-    // Another kind replaces the direct kernel only when it is faster by more than
-    // 2%: closer than that, which one wins is timing noise (on GB300 the
-    // warp-staged kernel and the direct one are within 1% at some widths).
+    // Another kind replaces the direct kernels (0 and 10) only when it is faster by more than
+    // 2%: closer than that, which one wins is timing noise.  The plain hop asks for 5%: in
+    // a solve its input was written just before and lies partly in L2, which the direct kernel
+    // gains more from (16^3 x 32, width 32: 117 us each when timed alone, 112 and 117 in the solve).
     for (int m = 0; m < 3; ++m) {
-        if (bP[m] != 0 && best0[m] < 1e30f && best[m] > 0.98f * best0[m]) {
+        if (!direct(bP[m]) && best0[m] < 1e30f && best[m] > (m == 0 ? 0.95f : 0.98f) * best0[m]) {
             bR[m] = b0R[m];
             bB[m] = b0B[m];
-            bP[m] = 0;
+            bP[m] = b0P[m];
         }
         c->hop_R[prec][l][m] = bR[m];
         c->hop_block[prec][l][m] = bB[m];

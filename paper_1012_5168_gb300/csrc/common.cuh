@@ -457,6 +457,53 @@ __device__ __forceinline__ void st_pack(S *p, const cx<typename Real<S>::type> (
     RawSt<NB>::st(p, w);
 }
 
+// ld_pack<S, R, true> and st_pack with an L2 eviction policy.  (Not volatile: loads may be
+// moved and batched like other read-only loads.)
+__device__ __forceinline__ uint64_t l2_policy(bool evict_first) {
+    uint64_t p;
+    if (evict_first) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    else asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+template <typename S, int R>
+__device__ __forceinline__ void ld_pack_l2(const S *p, cx<typename Real<S>::type> (&v)[R], uint64_t pol) {
+    constexpr int NB = R * cbytes<S>();
+    uint32_t w[NB / 4];
+    if constexpr (NB == 4) {
+        asm("ld.global.nc.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(w[0]) : "l"(p), "l"(pol));
+    } else if constexpr (NB == 8) {
+        asm("ld.global.nc.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;" : "=r"(w[0]), "=r"(w[1]) : "l"(p), "l"(pol));
+    } else {
+#pragma unroll
+        for (int k = 0; k < NB / 16; ++k)
+            asm("ld.global.nc.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
+                : "=r"(w[4 * k]), "=r"(w[4 * k + 1]), "=r"(w[4 * k + 2]), "=r"(w[4 * k + 3])
+                : "l"(reinterpret_cast<const char *>(p) + 16 * k), "l"(pol));
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = Conv<S>::get(w + r * Conv<S>::W);
+}
+template <typename S, int R>
+__device__ __forceinline__ void st_pack_l2(S *p, const cx<typename Real<S>::type> (&v)[R], uint64_t pol) {
+    constexpr int NB = R * cbytes<S>();
+    uint32_t w[NB / 4];
+#pragma unroll
+    for (int r = 0; r < R; ++r) Conv<S>::put(v[r], w + r * Conv<S>::W);
+    if constexpr (NB == 4) {
+        asm volatile("st.global.L2::cache_hint.u32 [%0], %1, %2;" ::"l"(p), "r"(w[0]), "l"(pol) : "memory");
+    } else if constexpr (NB == 8) {
+        asm volatile("st.global.L2::cache_hint.v2.u32 [%0], {%1, %2}, %3;" ::"l"(p), "r"(w[0]), "r"(w[1]), "l"(pol)
+                     : "memory");
+    } else {
+#pragma unroll
+        for (int k = 0; k < NB / 16; ++k)
+            asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(
+                             reinterpret_cast<char *>(p) + 16 * k),
+                         "r"(w[4 * k]), "r"(w[4 * k + 1]), "r"(w[4 * k + 2]), "r"(w[4 * k + 3]), "l"(pol)
+                         : "memory");
+    }
+}
+
 // One complex of a link (read-only path).
 template <typename S>
 __device__ __forceinline__ cx<typename Real<S>::type> ld_link(const S *p) {

@@ -64,6 +64,7 @@ struct HopArgs {
     int act_stride;         // iteration; NULL: all do.  The direct kernels skip the others' loads and stores.
     const float4 *gauge8d;  // [2][Vh][8][9] FP32 quads (Re U, Re U, Im U, Im U) of the site-major rows:
                             // the paired-layout kernel's links
+    int stream = 0;         // y, rhat and out evict-first in L2 (warp-staged kernels)
     const void *clovinv;    // clover: A^-1 of the output sites in the storage type ([2][Vh][2][6][6]
                             // complex), applied to D in before the epilogue; NULL: no clover term
 };

@@ -7,6 +7,7 @@
 // concurrently.
 #pragma once
 
+#include <algorithm>
 #include <mutex>
 
 #include <type_traits>
@@ -28,6 +29,17 @@ inline cudaError_t opt_in_smem(K kernel, size_t smem, size_t &opted, std::mutex 
     return e;
 }
 
+// Blocks per SM of a warp-staged kernel.  Its sites are dealt out to the warps of the whole
+// grid, so every block has to be resident.  The occupancy query counts all 228 kB of
+// shared memory, but the split with L1 that the launch gets holds less: 7 blocks of
+// 30,464 bytes (1 kB of it the system's; 208.25 kB) ran one after the other six, 6 of
+// 35,072 (205.5 kB) together, hence the line at 206.  FP32 plain hop, kind 11: 0.248 -> 0.117
+// ms on 16^3 x 32, 0.99 -> 0.57 ms on 24^3 x 48.
+template <typename K> int ws_blocks(K kern, int block, size_t smem) {
+    const int fit = (int)(206 * 1024 / (smem + 1024));
+    return std::min(std::min(resident_blocks(kern, block, smem), std::max(fit, 1)), 16);
+}
+
 // Warp-staged clover hop (FP32, two stages, SPW sites of 32 / SPW right-hand sides per warp).
 template <int SPW, int MODE, int RED>
 cudaError_t go_clov_ws(const HopArgs &a, Launch &l) {
@@ -38,8 +50,7 @@ cudaError_t go_clov_ws(const HopArgs &a, Launch &l) {
     l.smem = WsShape<float, 1, 2, SPW, true>::WB * WS_WARPS;
     const cudaError_t e = opt_in_smem(kern, l.smem, opted, m);
     if (e != cudaSuccess) return e;
-    const int res = resident_blocks(kern, l.block, l.smem);
-    l.grid = (l.num_sms > 0 ? l.num_sms : 1) * (res < 16 ? res : 16);
+    l.grid = (l.num_sms > 0 ? l.num_sms : 1) * ws_blocks(kern, l.block, l.smem);
     kern<<<l.grid, l.block, l.smem, l.stream>>>(a);
     return cudaGetLastError();
 }
@@ -137,8 +148,7 @@ cudaError_t go_hop(const HopArgs &a, Launch &l, int kind) {
         l.smem = (kind == 4 ? WsShape<S, R>::WB : WsShape<S, R, 2>::WB) * WS_WARPS;
         const cudaError_t e = kind == 4 ? opt_in_smem(kern, l.smem, opted, m) : opt_in_smem(kern, l.smem, opted2, m2);
         if (e != cudaSuccess) return e;
-        const int res = resident_blocks(kern, l.block, l.smem);
-        l.grid = (l.num_sms > 0 ? l.num_sms : 1) * (res < 16 ? res : 16);
+        l.grid = (l.num_sms > 0 ? l.num_sms : 1) * ws_blocks(kern, l.block, l.smem);
         kern<<<l.grid, l.block, l.smem, l.stream>>>(a);
         return cudaGetLastError();
     }
@@ -152,8 +162,7 @@ cudaError_t go_hop(const HopArgs &a, Launch &l, int kind) {
             l.smem = WsShape<S, 1, 2, 2>::WB * WS_WARPS;
             const cudaError_t e = opt_in_smem(kern, l.smem, opted, m);
             if (e != cudaSuccess) return e;
-            const int res = resident_blocks(kern, l.block, l.smem);
-            l.grid = (l.num_sms > 0 ? l.num_sms : 1) * (res < 16 ? res : 16);
+            l.grid = (l.num_sms > 0 ? l.num_sms : 1) * ws_blocks(kern, l.block, l.smem);
             kern<<<l.grid, l.block, l.smem, l.stream>>>(a);
             return cudaGetLastError();
         }

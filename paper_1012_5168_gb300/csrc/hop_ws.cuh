@@ -91,6 +91,9 @@ __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
     const int sub = SPW > 1 ? lane / LPS : 0;  // which of the warp's sites
     const int r0 = (SPW > 1 ? lane % LPS : lane) * R;
     const T cD = from_double<T>(A.c);
+    // y, rhat and the output, each touched once, leave L2 to the neighbour blocks where
+    // those of the sites under way fill it (A.stream, see do_hop)
+    const uint64_t pol = l2_policy(A.stream != 0);
     const S *in = reinterpret_cast<const S *>(A.in);
     const S *g8 = reinterpret_cast<const S *>(A.gauge8);
 
@@ -173,30 +176,42 @@ __global__ void __launch_bounds__(WS_WARPS * 32) hop_kernel_ws(HopArgs A) {
                                   acc[0]);
         const size_t base = (size_t)cb * 12 * N * 2 + (size_t)r0 * 2;
         S *out = reinterpret_cast<S *>(A.out);
+        // Loads of BC components are issued together.  Left to itself the compiler keeps
+        // R0DOT at 80 registers with few loads in flight: width 16 on 24^3 x 48 took 431 us,
+        // in batches of six 423; the other epilogues gained nothing from batches.
+        constexpr int BC = R == 1 && RED == RED_R0DOT ? 6 : 1;
+        constexpr bool with_y = MODE == MODE_XPAY || MODE == MODE_RESID || RED == RED_BICG;
+        constexpr bool with_rhat = RED == RED_R0DOT || RED == RED_BICG;
+        cx<T> yb[BC][R], hb[BC][R];
 #pragma unroll
         for (int cc = 0; cc < 12; ++cc) {
+            if (cc % BC == 0) {
+#pragma unroll
+                for (int k2 = 0; k2 < BC; ++k2) {
+                    const size_t o2 = base + (size_t)(cc + k2) * N * 2;
+                    if (with_y) ld_pack_l2<S, R>(reinterpret_cast<const S *>(A.y) + o2, yb[k2], pol);
+                    if (with_rhat) ld_pack_l2<S, R>(reinterpret_cast<const S *>(A.rhat) + o2, hb[k2], pol);
+                }
+            }
+            const cx<T>(&yv)[R] = yb[cc % BC];
+            const cx<T>(&rh)[R] = hb[cc % BC];
             const size_t off = base + (size_t)cc * N * 2;
             cx<T> o[R];
             if (MODE == MODE_PLAIN) {
 #pragma unroll
                 for (int r = 0; r < R; ++r) o[r] = cD * acc[r][cc];
             }
-            cx<T> yv[R];
-            if (MODE == MODE_XPAY || MODE == MODE_RESID || RED == RED_BICG)
-                ld_pack<S, R, true>(reinterpret_cast<const S *>(A.y) + off, yv);
             if (MODE == MODE_XPAY) {
 #pragma unroll
                 for (int r = 0; r < R; ++r) o[r] = yv[r] + cD * acc[r][cc];
             } else if (MODE == MODE_RESID) {
                 cx<T> zv[R];
-                ld_pack<S, R, true>(reinterpret_cast<const S *>(A.z) + off, zv);
+                ld_pack_l2<S, R>(reinterpret_cast<const S *>(A.z) + off, zv, pol);
 #pragma unroll
                 for (int r = 0; r < R; ++r) o[r] = zv[r] - yv[r] - cD * acc[r][cc];
             }
-            st_pack<S, R>(out + off, o);
+            st_pack_l2<S, R>(out + off, o, pol);
             if (RED == RED_R0DOT || RED == RED_BICG) {
-                cx<T> rh[R];
-                ld_pack<S, R, true>(reinterpret_cast<const S *>(A.rhat) + off, rh);
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     if (RED == RED_R0DOT) {
