@@ -111,7 +111,10 @@ typedef struct dl_solve_params {
     int batch;           /* right-hand sides solved together per launch (1..64, a power
                             of two for F32/BF16 >= 2); <= 0 picks 16 */
     int use_graph;       /* capture the inner iteration in CUDA graphs (1) or launch
-                            directly (0) */
+                            directly (0).  Small lattices (FP32 or BF16 inner, no
+                            clover, no timing, launch shape not pinned) run a whole
+                            inner cycle in one launch instead; this and chunk then
+                            have nothing to do */
     int chunk;           /* inner iterations per graph launch / convergence poll; <= 0: 2 */
     int method;          /* DL_METHOD_*; 0 (BiCGStab) by default */
 } dl_solve_params;
@@ -344,8 +347,8 @@ int dl_dilution_error(dl_ctx *ctx, uint64_t seed, int n_noise, unsigned dilution
  * ints, or NULL) restricts pair j to one timeslice; otherwise all T
  * timeslices are used.  Consecutive runs of `group` (1..64, dividing n_rhs)
  * pairs are summed.  host_out: double [n_rhs/group][n_sinks][n_mom][16][T][2].
- * The device work is a per-site spin matrix, its Fourier sum over each
- * timeslice (FP64, fixed order) and the Gamma traces.  Errors: DL_EINVAL for
+ * The device work is a spin matrix per site, summed over the group's pairs, its
+ * Fourier sum over each timeslice (FP64, fixed order) and the Gamma traces.  Errors: DL_EINVAL for
  * bad arguments, DL_ESTATE without a gauge field for the smeared sink,
  * DL_ENOMEM, DL_ECUDA. */
 int dl_trace_loops_mom(dl_ctx *ctx, const void *dev_eta, const void *dev_phi, int n_rhs, int sink,
@@ -362,7 +365,7 @@ int dl_trace_loops_mom(dl_ctx *ctx, const void *dev_eta, const void *dev_phi, in
  * and dl_solve).  host_out: double [n_mom][16 A][16 B][T][2] for all source
  * (A) and sink (B) operators of the Gamma basis.  For A = B = gamma5 (the
  * pion) the value is -sum_x Tr[S^dag S] < 0 in this sign convention.
- * Allocates 4 KiB per lattice site of scratch device memory (kept by the
+ * Allocates 2176 bytes per lattice site of scratch device memory (kept by the
  * context). */
 int dl_meson_correlators(dl_ctx *ctx, const void *dev_prop, const int src[4], const int *momenta, int n_mom,
                          double *host_out);
