@@ -40,7 +40,7 @@ constexpr int WS_WARPS = 4;  // warps per block of the warp-staged hop
 // latency, small enough that four 4-warp blocks fit in one SM's shared memory.
 // NSTO = 2 (kernel kind 11) keeps one copy in flight and so fits about twice
 // the warps per SM: on GB300 that runs the fused hops faster (their epilogue
-// loads gain from the extra warps) and the plain hop slower.
+// loads gain from the extra warps) and the plain hop at the direct kernel's speed.
 template <typename S, int R, int NSTO = 0, int SPW = 1, bool CLOV = false>
 struct WsShape {
     static constexpr uint32_t SB = 12u * 32u * R * cbytes<S>();  // SPW neighbour blocks [12][N], N = 32 R / SPW
