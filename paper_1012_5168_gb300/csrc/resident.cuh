@@ -132,7 +132,8 @@ __device__ __forceinline__ void res_bar(int grp) { asm volatile("bar.sync %0, 12
 
 // The NV complex sums over the cluster of the threads' red[], into sh.total of
 // every block, in a fixed order: lanes, warps (four runs), ranks (four runs).
-// Contains the cluster barrier that also orders the phase's field stores.
+// Contains the cluster barrier that also orders the phase's field stores.  With C > 1 it
+// writes into the other blocks' shared memory: a cluster barrier must lie before the first call.
 template <int NV, typename T>
 __device__ __forceinline__ void res_sum(ResShared<T> &sh, cx<T> (&red)[NV], int C, int rank, int buf) {
     const int tid = threadIdx.x, lane = tid & 31;
@@ -280,6 +281,10 @@ __global__ void __launch_bounds__(RES_THREADS, 1) resident_kernel(ResArgs A) {
         }
         res_bar(grp);
     };
+
+    // A block's shared memory may be written from another block only once it has started, and
+    // the set-up's res_sum is the first to do so.
+    if (C > 1) cluster.sync();
 
     // ---- phase set-up: fields from the FP64 residual
     const OuterState &o = A.os[rg];
