@@ -287,10 +287,9 @@ static int do_hop(dl_ctx *c, int prec, int mode, int red, void *out, const void 
                                 : (const void *)c->d_clovinv16;
     // Evict-first for the streams once a timeslice of the input exceeds 8 MB: the hop reuses
     // three of them, and a line read from both dies takes its place in both halves of L2.
-    // 24^3 x 48, FP32, width 32 (21 MB): the fused hops from 0.906 and 0.907 to 0.761 and
-    // 0.770 ms; width 16 (10.6 MB): the same within 1%.  16^3 x 32, width 32 (6.3 MB): the
-    // hops alone the same, a solve 0.7% slower with it, since the vector updates find less
-    // of v, s and t in L2.
+    // 24^3 x 48, FP32, width 32 (21 MB): the fused hops from 0.907 to 0.777 ms; width 16
+    // (10.6 MB): 420 to 406 us.  16^3 x 32, width 32 (6.3 MB): the hops alone the same, a
+    // solve 0.7% slower with it, since the vector updates find less of v, s and t in L2.
     a.stream = (size_t)c->g.V3h * 24 * N * storage_bytes(prec) > ((size_t)8 << 20);
     const int m = hop_class(mode, red);  // the shape tables' entry
     int R = (wide || clov) ? 1 : c->hop_R[prec][ilog2(N)][m];

@@ -459,10 +459,9 @@ __device__ __forceinline__ void st_pack(S *p, const cx<typename Real<S>::type> (
 
 // ld_pack<S, R, true> and st_pack with an L2 eviction policy.  (Not volatile: loads may be
 // moved and batched like other read-only loads.)
-__device__ __forceinline__ uint64_t l2_policy(bool evict_first) {
+__device__ __forceinline__ uint64_t l2_evict_first() {
     uint64_t p;
-    if (evict_first) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-    else asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
 template <typename S, int R>

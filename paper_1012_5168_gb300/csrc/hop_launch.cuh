@@ -30,29 +30,43 @@ inline cudaError_t opt_in_smem(K kernel, size_t smem, size_t &opted, std::mutex 
 }
 
 // Blocks per SM of a warp-staged kernel.  Its sites are dealt out to the warps of the whole
-// grid, so every block has to be resident.  The occupancy query counts all 228 kB of
-// shared memory, but the split with L1 that the launch gets holds less: 7 blocks of
-// 30,464 bytes (1 kB of it the system's; 208.25 kB) ran one after the other six, 6 of
-// 35,072 (205.5 kB) together, hence the line at 206.  FP32 plain hop, kind 11: 0.248 -> 0.117
-// ms on 16^3 x 32, 0.99 -> 0.57 ms on 24^3 x 48.
+// grid, so every block has to be resident.  The occupancy query counts all 228 kB of shared
+// memory, but the launch may be given the next smaller split with L1, 196 kB.  Which one
+// follows from how much of the larger split's blocks the smaller one holds: with 6 of 7
+// (plain hop, FP32, kind 11, width 32: seven blocks of 30,464 bytes, 1 kB of it the system's) six ran together,
+// the seventh after them (0.248 ms on 16^3 x 32 against 0.121 with six); with 5 of 6 (kind
+// 12) and 3 of 4 (kind 4 at width 32, kind 11 at width 64: 94 us against 100 with three
+// on 16 x 20 x 8 x 22) the larger one.  Hence the line at 0.85.
 template <typename K> int ws_blocks(K kern, int block, size_t smem) {
-    const int fit = (int)(206 * 1024 / (smem + 1024));
+    const int small = (int)(196 * 1024 / (smem + 1024)), large = (int)(228 * 1024 / (smem + 1024));
+    const int fit = 20 * small >= 17 * large ? small : large;
     return std::min(std::min(resident_blocks(kern, block, smem), std::max(fit, 1)), 16);
 }
 
-// Warp-staged clover hop (FP32, two stages, SPW sites of 32 / SPW right-hand sides per warp).
-template <int SPW, int MODE, int RED>
-cudaError_t go_clov_ws(const HopArgs &a, Launch &l) {
+// Warp-staged hop (hop_ws.cuh): NSTO stages (0: as many as suit the width), SPW sites of 32 R / SPW
+// right-hand sides per warp.  Evict-first streams (a.stream) in FP32 where they gain: 24^3 x 48,
+// width 32, fused hops of kinds 4 and 11 907 -> 842 and 907 -> 777 us, plain hop of kind 11
+// 581 -> 570; width 16 (kind 12) fused 420 -> 406, plain 303 -> 305; 24 x 16 x 8 x 40, width 64,
+// fused 282 -> 275, plain 194 both.  BF16: 843 -> 847 and 920 -> 938 fused.
+template <typename S, int R, int MODE, int RED, int NSTO, int SPW, bool CLOV, bool EF>
+cudaError_t go_ws_ef(const HopArgs &a, Launch &l) {
     static size_t opted = 0;
     static std::mutex m;
-    auto kern = hop_kernel_ws<float, 1, MODE, RED, 2, SPW, true>;
+    auto kern = hop_kernel_ws<S, R, MODE, RED, NSTO, SPW, CLOV, EF>;
     l.block = WS_WARPS * 32;
-    l.smem = WsShape<float, 1, 2, SPW, true>::WB * WS_WARPS;
+    l.smem = WsShape<S, R, NSTO, SPW, CLOV>::WB * WS_WARPS;
     const cudaError_t e = opt_in_smem(kern, l.smem, opted, m);
     if (e != cudaSuccess) return e;
     l.grid = (l.num_sms > 0 ? l.num_sms : 1) * ws_blocks(kern, l.block, l.smem);
     kern<<<l.grid, l.block, l.smem, l.stream>>>(a);
     return cudaGetLastError();
+}
+template <typename S, int R, int MODE, int RED, int NSTO, int SPW = 1, bool CLOV = false>
+cudaError_t go_ws(const HopArgs &a, Launch &l) {
+    if (a.N != 32 * R / SPW) return cudaErrorInvalidValue;
+    if constexpr (std::is_same<S, float>::value && (RED != RED_NONE || (R == 1 && SPW == 1 && NSTO == 2)))
+        if (a.stream) return go_ws_ef<S, R, MODE, RED, NSTO, SPW, CLOV, true>(a, l);
+    return go_ws_ef<S, R, MODE, RED, NSTO, SPW, CLOV, false>(a, l);
 }
 
 template <typename S, int R, int MODE, int RED>
@@ -63,8 +77,8 @@ cudaError_t go_hop(const HopArgs &a, Launch &l, int kind) {
             // width 32: 136 us plain, 158 and 173 fused, where the direct kernel with its
             // 1152 bytes of links and A^-1 per thread took 147, 203 and 216.
             if constexpr (std::is_same<S, float>::value) {
-                if (a.N == 32) return go_clov_ws<1, MODE, RED>(a, l);
-                if (a.N == 16) return go_clov_ws<2, MODE, RED>(a, l);
+                if (a.N == 32) return go_ws<S, 1, MODE, RED, 2, 1, true>(a, l);
+                if (a.N == 16) return go_ws<S, 1, MODE, RED, 2, 2, true>(a, l);
             }
             clamp_grid(l, resident_blocks(hop_kernel_clov<S, MODE, RED>, l.block, l.smem));
             hop_kernel_clov<S, MODE, RED><<<l.grid, l.block, l.smem, l.stream>>>(a);
@@ -139,33 +153,10 @@ cudaError_t go_hop(const HopArgs &a, Launch &l, int kind) {
         direct<<<l.grid, l.block, l.smem, l.stream>>>(b);
         return cudaGetLastError();
     }
-    if (kind == 4 || kind == 11) {  // warp-staged: one site per warp, so N = 32 R; kind 11 with two stages
-        if (a.N != 32 * R) return cudaErrorInvalidValue;
-        static size_t opted = 0, opted2 = 0;
-        static std::mutex m, m2;
-        auto kern = kind == 4 ? hop_kernel_ws<S, R, MODE, RED> : hop_kernel_ws<S, R, MODE, RED, 2>;
-        l.block = WS_WARPS * 32;
-        l.smem = (kind == 4 ? WsShape<S, R>::WB : WsShape<S, R, 2>::WB) * WS_WARPS;
-        const cudaError_t e = kind == 4 ? opt_in_smem(kern, l.smem, opted, m) : opt_in_smem(kern, l.smem, opted2, m2);
-        if (e != cudaSuccess) return e;
-        l.grid = (l.num_sms > 0 ? l.num_sms : 1) * ws_blocks(kern, l.block, l.smem);
-        kern<<<l.grid, l.block, l.smem, l.stream>>>(a);
-        return cudaGetLastError();
-    }
-    if (kind == 12) {  // warp-staged at width 16, two sites per warp (FP32), two stages
-        if constexpr (std::is_same<S, float>::value && R == 1) {
-            if (a.N != 16) return cudaErrorInvalidValue;
-            static size_t opted = 0;
-            static std::mutex m;
-            auto kern = hop_kernel_ws<S, 1, MODE, RED, 2, 2>;
-            l.block = WS_WARPS * 32;
-            l.smem = WsShape<S, 1, 2, 2>::WB * WS_WARPS;
-            const cudaError_t e = opt_in_smem(kern, l.smem, opted, m);
-            if (e != cudaSuccess) return e;
-            l.grid = (l.num_sms > 0 ? l.num_sms : 1) * ws_blocks(kern, l.block, l.smem);
-            kern<<<l.grid, l.block, l.smem, l.stream>>>(a);
-            return cudaGetLastError();
-        }
+    if (kind == 4) return go_ws<S, R, MODE, RED, 0>(a, l);  // warp-staged: one site per warp, so N = 32 R
+    if (kind == 11) return go_ws<S, R, MODE, RED, 2>(a, l);  // the same with two stages
+    if (kind == 12) {  // at width 16, two sites per warp (FP32), two stages
+        if constexpr (std::is_same<S, float>::value && R == 1) return go_ws<S, 1, MODE, RED, 2, 2>(a, l);
         return cudaErrorInvalidValue;
     }
     if (kind == 6) {  // direct loads, packed FP32 arithmetic (FP32 storage, R = 1)
