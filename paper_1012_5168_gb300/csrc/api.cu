@@ -784,7 +784,8 @@ extern "C" int dl_create(dl_ctx **out, const int dims[4], int t_bc, void *cuda_s
     if (rc == DL_OK) c->h_err[0] = c->h_err[1] = 0;
     if (rc == DL_OK &&
         (cudaMemcpy(c->d_coords, coords.data(), V * sizeof(uint32_t), cudaMemcpyHostToDevice) != cudaSuccess ||
-         cudaMemcpy(c->d_gammas, gh.data(), 256 * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess))
+         cudaMemcpy(c->d_gammas, gh.data(), 256 * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess ||
+         cudaMemsetAsync(c->d_smear, 0, sizeof(SmearList), c->stream) != cudaSuccess))
         rc = fail(DL_ECUDA, "context upload failed");
     if (rc != DL_OK) {
         dl_destroy(c);
@@ -1807,34 +1808,44 @@ static int smear_eo(dl_ctx *c, double **buf, double *spare, int N, int n, const 
     } else {
         double *src2 = buf2 ? *buf2 : nullptr, *dst2 = spare2;
         const int nf = buf2 ? 2 : 1;
-        SmearList *L = c->d_smear;
-        CK(cudaMemsetAsync(L, 0, offsetof(SmearList, g), c->cur));
-        Launch lf = make_launch(c, 2L * (cb1 - cb0) * n, 256, 0, 8);
-        Launch lc = make_launch(c, 2L * (cb1 - cb0) * 12 * n, 256, 0, 8);
-        for (int f = 0; f < nf; ++f) {
-            double *x = f ? src2 : src;
-            smear_flags_kernel<<<lf.grid, lf.block, 0, c->cur>>>(x, (int)c->Vh, cb0, cb1, N, n, tcol, c->g.V3h,
-                                                                 L->flags[f]);
-            ff_convert_kernel<<<lc.grid, lc.block, 0, c->cur>>>(x, (int)c->Vh, cb0, cb1, N, n, 1, tcol, c->g.V3h,
-                                                                nullptr);
-        }
-        smear_list_kernel<<<1, 64, 0, c->cur>>>(L, n, nf, tcol);
-        // one thread per (site, colour row, group of columns), sized for dense fields; the
-        // list's length is known on the device only
+        // Where the dense groups (the four spins of a right-hand side) give no SM a second block,
+        // leaving out zero spins gains nothing, and finding them costs three launches' latency and a step's
+        // threads one more dependent load: 4 x 4 x 6, 24 pairs: 668 us without a list, 698 with one;
+        // 4 x 22 x 4 (198 blocks): 926 and 757.
         Launch lr = make_launch(c, 2L * (cb1 - cb0) * 3 * n * nf, 256, 0, 64);
+        SmearList *L = lr.grid > c->num_sms ? c->d_smear : nullptr;
+        Launch lc = make_launch(c, 2L * (cb1 - cb0) * 12 * n, 256, 0, 8);
+        if (L) {
+            Launch lf = make_launch(c, 2L * (cb1 - cb0) * n, 256, 0, 8);
+            smear_flags_kernel<<<dim3(lf.grid, nf), lf.block, 0, c->cur>>>(src, src2, (int)c->Vh, cb0, cb1, N, n, tcol,
+                                                                          c->g.V3h, L);
+            smear_list_kernel<<<1, 64, 0, c->cur>>>(L, n, nf, tcol);
+            c->kernel_launches += 2;
+        }
+        for (int f = 0; f < nf; ++f)
+            ff_convert_kernel<<<lc.grid, lc.block, 0, c->cur>>>(f ? src2 : src, (int)c->Vh, cb0, cb1, N, n, 1, tcol,
+                                                                c->g.V3h, nullptr);
+        // one thread per (site, colour row, group of columns), sized for dense fields; the list's
+        // length is known on the device only.  A grid that is resident at once (two blocks per SM)
+        // spreads the list over all SMs: 22 x 6 x 4 (297 blocks), 24 pairs, 918 us; 971 without a
+        // list, 979 to 1009 with the list in the first blocks.
+        const bool spread = L && lr.grid <= 2 * c->num_sms;
+        if (spread) lr.grid = 2 * c->num_sms;
         for (int it = 0; it < s.n_iter; ++it) {
             A.in = src;
             A.out = dst;
             A.in2 = src2;
             A.out2 = dst2;
-            smear_ff_rows_kernel<<<lr.grid, lr.block, 0, c->cur>>>(A, c->d_gauge_ff, L);
+            auto step = !L ? smear_ff_rows_kernel<false, false>
+                           : (spread ? smear_ff_rows_kernel<true, true> : smear_ff_rows_kernel<true, false>);
+            step<<<lr.grid, lr.block, 0, c->cur>>>(A, c->d_gauge_ff, L, nf);
             std::swap(src, dst);
             std::swap(src2, dst2);
         }
         for (int f = 0; f < nf; ++f)
             ff_convert_kernel<<<lc.grid, lc.block, 0, c->cur>>>(f ? src2 : src, (int)c->Vh, cb0, cb1, N, n, 0, tcol,
-                                                                c->g.V3h, &L->flags[f][0][0]);
-        c->kernel_launches += s.n_iter + 3 * nf + 1;
+                                                                c->g.V3h, L ? &L->flags[f][0][0] : nullptr);
+        c->kernel_launches += s.n_iter + 2 * nf;
         if (buf2) *buf2 = src2;
     }
     CK(cudaGetLastError());

@@ -438,7 +438,7 @@ __device__ __forceinline__ ffc ld_ffc(const double *p) {
 
 // In-place conversion of an EO tile field (both parities, cb range, n of N
 // columns) between FP64 and float-float.  to_ff = 1: double -> ff; 0: back.
-// flags (back only): spins flags[j][s] == 0 were left out of the iterations and become 0.
+// flags (back only, may be NULL): spins flags[j][s] == 0 were left out of the iterations and become 0.
 static __global__ void ff_convert_kernel(double *f, int Vh, int cb0, int cb1, int N, int n, int to_ff,
                                          const int *tcol, int V3h, const int *flags) {
     const long nsite = cb1 - cb0;
@@ -458,7 +458,7 @@ static __global__ void ff_convert_kernel(double *f, int Vh, int cb0, int cb1, in
             const float4 v = *reinterpret_cast<const float4 *>(e);
             ff a, b;
             a.hi = v.x; a.lo = v.y; b.hi = v.z; b.lo = v.w;
-            const bool on = flags[j * 4 + c / 3] != 0;
+            const bool on = !flags || flags[j * 4 + c / 3] != 0;
             e[0] = on ? (double)a : 0.0;
             e[1] = on ? (double)b : 0.0;
         }
@@ -486,13 +486,16 @@ struct SmearGroup {
 };
 struct SmearList {
     int n_groups;
+    int found[2][64][4];  // all zero between smearings
     int flags[2][64][4];
     SmearGroup g[128];
 };
 
-// flags of one field (cleared before): blocks over sites, right-hand sides fastest.
-static __global__ void smear_flags_kernel(const double *f, int Vh, int cb0, int cb1, int N, int n, const int *tcol,
-                                          int V3h, int (*flags)[4]) {
+// found[field] of the fields blockIdx.y = 0 (f0) and 1 (f1): blocks over sites, right-hand sides fastest.
+static __global__ void smear_flags_kernel(const double *f0, const double *f1, int Vh, int cb0, int cb1, int N, int n,
+                                          const int *tcol, int V3h, SmearList *L) {
+    const double *f = blockIdx.y ? f1 : f0;
+    int(*flags)[4] = L->found[blockIdx.y];
     const long nsite = cb1 - cb0, total = 2 * nsite * n;
     for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
         const int j = (int)(idx % n);
@@ -517,7 +520,10 @@ static __global__ void smear_flags_kernel(const double *f, int Vh, int cb0, int 
 static __global__ void smear_list_kernel(SmearList *L, int n, int nf, const int *tcol) {
     __shared__ int flags[2][64][4], ts[64], count[2];
     __shared__ SmearGroup g[2][64];
-    for (int k = threadIdx.x; k < 512; k += 64) flags[k >> 8][(k >> 2) & 63][k & 3] = L->flags[k >> 8][(k >> 2) & 63][k & 3];
+    for (int k = threadIdx.x; k < 512; k += 64) {
+        (&flags[0][0][0])[k] = (&L->flags[0][0][0])[k] = (&L->found[0][0][0])[k];
+        (&L->found[0][0][0])[k] = 0;
+    }
     if ((int)threadIdx.x < n) ts[threadIdx.x] = tcol ? tcol[threadIdx.x] : 0;
     __syncthreads();
     if ((int)threadIdx.x < 2) {
@@ -560,19 +566,33 @@ static __global__ void smear_list_kernel(SmearList *L, int n, int nf, const int 
 // thread) measured 9% faster than three (85).  48 pairs of spin-diluted sources
 // and solutions on one 16^3 timeslice: 114 us a step with the groups, 176 us
 // on all 384 columns.
+// Without a list (LIST false) the groups are the four spins of each right-hand side of nf fields.
+// SPREAD: the grid holds more threads than there is work, and all its blocks take an equal part.
+template <bool LIST, bool SPREAD>
 static __global__ void __launch_bounds__(256, 2) smear_ff_rows_kernel(SmearArgs A, const float *gauge_ff,
-                                                                      const SmearList *L) {
-    const int nsite = A.cb1 - A.cb0, ng = L->n_groups;
+                                                                      const SmearList *L, int nf) {
+    const int nsite = A.cb1 - A.cb0, ng = LIST ? L->n_groups : A.n * nf;
     const long total = 2L * nsite * 3 * ng;
     const size_t half = (size_t)A.g.Vh * 12 * A.N * 2;
     const ff fa = df_from_double(A.a), fc = df_from_double(A.c);
-    for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
+    const int per = SPREAD ? (int)((total + gridDim.x - 1) / gridDim.x + 31) & ~31 : blockDim.x;
+    if (SPREAD && (int)threadIdx.x >= per) return;
+    for (long idx = (long)blockIdx.x * per + threadIdx.x; idx < total; idx += (long)gridDim.x * per) {
         const int gi = (int)(idx % ng);
         const long rest = idx / ng;
         const int a = (int)(rest % 3);
         const int sp = (int)(rest / 3);
         const int p = sp / nsite;
-        const SmearGroup G = L->g[gi];
+        SmearGroup G;
+        if (LIST) {
+            G = L->g[gi];
+        } else {
+            const int j = gi % A.n;
+            G.field = gi / A.n;
+            G.t = A.tcol ? A.tcol[j] : 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) G.col[k] = j << 2 | k;
+        }
         const double *__restrict__ fin = G.field ? A.in2 : A.in;
         double *__restrict__ fout = G.field ? A.out2 : A.out;
         const int cb = A.cb0 + sp % nsite + (A.tcol ? G.t * A.g.V3h : 0);
