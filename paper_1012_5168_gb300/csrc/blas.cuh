@@ -57,22 +57,34 @@ struct OuterState {
 // (by the exponent bits: a comparison would be one more FP64 instruction)
 __device__ __forceinline__ bool finite1(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 __device__ __forceinline__ bool finite2(double2 z) { return finite1(z.x) && finite1(z.y); }
-// 1/x by the hardware's approximation and two Newton steps.  On GB300 an FP64
-// instruction of a warp takes about 70 cycles, whatever its lanes do, and an
-// IEEE division 750 to 1500 (measured: 8 dependent divisions 12,400 cycles, 8 of
-// these reciprocals 3,100); the scalar recurrences below sit on every iteration's
-// critical path.
+// 1/x for 2^-1020 <= |x| < 2^1020 by the hardware's approximation (about 20 bits) and two Newton
+// steps, each of which squares the relative error: what is left is rounding, within 2^-52 of
+// 1/x.  On GB300 an FP64 instruction of a warp takes about 70 cycles, whatever its
+// lanes do, and an IEEE division 750 to 1500 (measured: 8 dependent divisions 12,400
+// cycles, 8 of these reciprocals 3,100); the scalar recurrences below sit on every
+// iteration's critical path.
 __device__ __forceinline__ double fp64_rcp(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     r = ::fma(r, ::fma(-x, r, 1.0), r);
     return ::fma(r, ::fma(-x, r, 1.0), r);
 }
+// The approximation takes a subnormal for zero and makes a subnormal result zero: outside
+// fp64_rcp's range, and for zeros, infinities and NaN, the quotients below divide.
+__device__ __forceinline__ bool rcp_in_range(double x) {
+    return (unsigned)(((__double2hiint(x) >> 20) & 0x7ff) - 3) < 2040u;  // biased exponent 3 .. 2042
+}
+__device__ __forceinline__ double fp64_div(double a, double b) { return rcp_in_range(b) ? a * fp64_rcp(b) : a / b; }
+__device__ __forceinline__ double2 fp64_div(double2 a, double b) {
+    if (!rcp_in_range(b)) return make_double2(a.x / b, a.y / b);
+    const double i = fp64_rcp(b);
+    return make_double2(a.x * i, a.y * i);
+}
 // a / b for b2 = |b|^2
 __device__ __forceinline__ double2 cdiv_by(double2 a, double2 b, double b2) {
-    const double i = fp64_rcp(b2);
-    return make_double2((a.x * b.x + a.y * b.y) * i, (a.y * b.x - a.x * b.y) * i);
+    return fp64_div(make_double2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y), b2);
 }
+__device__ __forceinline__ double2 cdiv(double2 a, double2 b) { return cdiv_by(a, b, b.x * b.x + b.y * b.y); }
 __device__ __forceinline__ double2 cmul2(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
@@ -219,7 +231,8 @@ __device__ __forceinline__ void bicg_omega(RhsState &s, const double2 (&v)[5]) {
         s.next_active = 0;
         return;
     }
-    if (!(tt > 0.0)) {
+    const double2 om = fp64_div(ts, tt);
+    if (!(tt > 0.0) || !finite2(om)) {
         // t = 0: s is already the solution's residual (zero) or the iteration broke down
         s.omega = make_double2(0.0, 0.0);
         s.r2 = ss;
@@ -227,16 +240,17 @@ __device__ __forceinline__ void bicg_omega(RhsState &s, const double2 (&v)[5]) {
         if (ss > s.target2) s.status = ST_BREAKDOWN;
         stop = true;
     } else {
-        const double it = fp64_rcp(tt);
-        const double2 om = make_double2(ts.x * it, ts.y * it);
         const double2 rho_new = make_double2(r0s.x - (om.x * r0t.x - om.y * r0t.y),
                                              r0s.y - (om.x * r0t.y + om.y * r0t.x));
         double r2 = ss - (ts.x * om.x + ts.y * om.y);
         if (r2 < 0.0) r2 = 0.0;
         s.omega = om;
         s.r2 = r2;
-        const double2 den = cmul2(s.rho, om);  // beta = (rho'/rho)(alpha/omega) with one reciprocal
-        const double2 beta = cdiv_by(cmul2(rho_new, s.alpha), den, den.x * den.x + den.y * den.y);
+        // beta = (rho'/rho)(alpha/omega), with one reciprocal where the product's square is in its range
+        const double2 den = cmul2(s.rho, om);
+        const double den2 = den.x * den.x + den.y * den.y;
+        const double2 beta = rcp_in_range(den2) ? cdiv_by(cmul2(rho_new, s.alpha), den, den2)
+                                                : cmul2(cdiv(rho_new, s.rho), cdiv(s.alpha, om));
         if (!finite2(beta) || !(rho_new.x * rho_new.x + rho_new.y * rho_new.y > 0.0)) {
             s.beta = make_double2(0.0, 0.0);
             if (r2 > s.target2) s.status = ST_BREAKDOWN;
@@ -253,7 +267,7 @@ __device__ __forceinline__ void bicg_omega(RhsState &s, const double2 (&v)[5]) {
 __device__ __forceinline__ void cg_alpha(RhsState &s, double ww) {
     s.active = s.next_active;
     if (!s.active) return;
-    const double a = s.rho.x * fp64_rcp(ww);
+    const double a = fp64_div(s.rho.x, ww);
     if (!(ww > 0.0) || !finite1(a)) {
         s.status = finite1(ww) ? ST_BREAKDOWN : ST_NAN;
         s.active = 0;
@@ -278,7 +292,7 @@ __device__ __forceinline__ void cg_beta(RhsState &s, double r2, double zz) {
         if (r2 > s.target2) s.status = ST_BREAKDOWN;
         stop = true;
     } else {
-        s.beta = make_double2(zz * fp64_rcp(s.rho.x), 0.0);
+        s.beta = make_double2(fp64_div(zz, s.rho.x), 0.0);
         s.rho = make_double2(zz, 0.0);
     }
     const bool done = s.fixed ? (s.iters >= s.max_iters) : (s.r2 <= s.target2 || s.iters >= s.max_iters);
