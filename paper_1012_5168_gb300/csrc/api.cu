@@ -134,7 +134,7 @@ struct dl_ctx {
     int *h_count = nullptr;  // pinned, mapped
     int *d_count = nullptr;
 
-    std::map<std::tuple<int, int, int, int>, GraphEntry> graphs;
+    std::map<std::tuple<int, int, int, int, int>, GraphEntry> graphs;
     bool timing = false;
     std::vector<TimedPair> pending;  // recorded eagerly, harvested at the next sync
     std::vector<cudaEvent_t> event_pool;
@@ -1128,7 +1128,7 @@ static int enqueue_iteration_cg(dl_ctx *c, int prec, int N) {
 // sides still active in *active.
 static int run_chunk(dl_ctx *c, int prec, int N, int iters, bool use_graph, int *active, int method) {
     if (use_graph) {
-        auto key = std::make_tuple(prec + 4 * method, N, iters, c->timing ? 1 : 0);
+        auto key = std::make_tuple(prec, method, N, iters, c->timing ? 1 : 0);
         auto it = c->graphs.find(key);
         if (it == c->graphs.end()) {
             GraphEntry ge;
