@@ -15,8 +15,8 @@ static cudaError_t go(const HopArgs &a, Launch &l) {
     }
     // Where every SM gets at most one block of 64 (site, right-hand side) items, four warps
     // share 32 of them (hop_split.cuh), one group a block while that fills no more than the
-    // SMs: plain hops of 12.4 us (up to 32 items an SM) and 18.5 us (64) against 31 us for
-    // any number of sites up to 100 an SM; at 108 items an SM both take 33 us.
+    // SMs: plain hops of 12.4 us (up to 32 items an SM) and 20.5 us (64) against 33 us for
+    // any number of sites up to 100 an SM; at 108 items an SM both take 35 us.
     const long items = (long)(a.cb_end - a.cb_begin) * a.N;
     if (l.num_sms > 0 && items <= 64L * l.num_sms) {
         const int groups = a.N <= 32 && items <= 32L * l.num_sms ? 1 : 2;
@@ -28,7 +28,7 @@ static cudaError_t go(const HopArgs &a, Launch &l) {
         return cudaGetLastError();
     }
     // 168 registers let six blocks of 64 threads share an SM (about 180: five).  One right-hand
-    // side on 16^3 x 32: 107 / 115 / 135 us (plain, <rhat, v>, five sums) against 116 / 125 / 144.
+    // side on 16^3 x 32: 115 / 121 / 141 us (plain, <rhat, v>, five sums) against 124 / 131 / 152.
     auto kernel = hop_kernel_cap<double, R, MODE, RED, 168>;
     clamp_grid(l, resident_blocks(kernel, l.block, l.smem));
     kernel<<<l.grid, l.block, l.smem, l.stream>>>(a);

@@ -1,12 +1,12 @@
 // The FP64 Wilson hop with the four direction pairs of an output site on four
 // warps, for launches with few sites.
 //
-// A whole-site thread issues about 820 FP64 instructions, one after the other at
+// A whole-site thread issues about 870 FP64 instructions, one after the other at
 // 17 to 70 cycles each (two FP64 lanes a clock and SM, about 70 cycles latency): a
 // launch that leaves an SM with few warps is bound by that chain, not by the
 // units.  Here warp q of four takes mu = q, forward and backward, of 32 (site,
 // right-hand side) items; the four contributions meet in shared memory, and warp q
-// goes on with spin q: 220 instructions a thread, a tenth more in all.  A block is
+// goes on with spin q: 230 instructions a thread, a twentieth more in all.  A block is
 // one such group or two (GR; width 64 needs two, for a thread to keep its
 // right-hand side).
 #pragma once
