@@ -178,9 +178,8 @@ int dl_set_kappa(dl_ctx *ctx, double kappa);
  * is still D alone.  The even-odd solve uses the asymmetric Schur system
  * A_ee^-1 (A_ee - kappa^2 D_eo A_oo^-1 D_oe) with A^-1 applied in the inner
  * hops; the residual and tolerance remain those of b - M x.  BiCGStab only:
- * a solve with DL_METHOD_CGNR fails with DL_EINVAL.  Mixed-precision clover solves
- * run their defect-correction steps in float-float arithmetic for tol >= 1e-11, as
- * without clover (another 2304 bytes per site for the blocks in that format).  Errors: DL_EINVAL
+ * a solve with DL_METHOD_CGNR fails with DL_EINVAL, and mixed-precision clover
+ * solves run their defect-correction steps in FP64.  Errors: DL_EINVAL
  * (non-finite c_sw), DL_ECUDA; an allocation failure (DL_ENOMEM) is reported
  * by the call that builds the blocks. */
 int dl_set_clover(dl_ctx *ctx, double c_sw);

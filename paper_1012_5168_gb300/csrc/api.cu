@@ -99,8 +99,6 @@ struct dl_ctx {
     double2 *d_clovinv64 = nullptr;  // A^-1 in FP64, FP32 and BF16
     float2 *d_clovinv32 = nullptr;
     bf16 *d_clovinv16 = nullptr;
-    float *d_clovff = nullptr;       // A, then A^-1, in float-float (mixed-precision solves)
-    bool clovff_ok = false;
 
     // batch workspace, width ws_N (power of two)
     int ws_N = 0;
@@ -809,7 +807,7 @@ extern "C" int dl_destroy(dl_ctx *c) {
                     c->d_gauge_ff, c->d_gammas,  c->d_partials, c->d_acc,     c->d_noise,     c->d_w,
                     c->d_smear,
                     c->d_reslinks[0], c->d_reslinks[1], c->d_reslinks[2],
-                    c->d_tcol,     c->d_acc2,    c->d_clov64,   c->d_clovinv64, c->d_clovinv32, c->d_clovinv16, c->d_clovff};
+                    c->d_tcol,     c->d_acc2,    c->d_clov64,   c->d_clovinv64, c->d_clovinv32, c->d_clovinv16};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (dl_ctx::Scratch *sc : {&c->s_phase, &c->s_site, &c->s_msum, &c->s_mloops, &c->s_mgroup, &c->s_mom,
@@ -949,30 +947,6 @@ static int ensure_clover(dl_ctx *c) {
                            reinterpret_cast<__nv_bfloat162 *>(c->d_clovinv16), grid, c->stream));
     c->kernel_launches++;
     c->clover_stale = false;
-    c->clovff_ok = false;
-    return DL_OK;
-}
-
-// Float-float copies of the clover blocks for the defect-correction steps of mixed precision.
-static int ensure_clover_ff(dl_ctx *c) {
-    if (c->clovff_ok) return DL_OK;
-    const size_t n = (size_t)c->V * 72;  // complex entries
-    if (!c->d_clovff && cudaMalloc((void **)&c->d_clovff, 2 * n * sizeof(float4)) != cudaSuccess)
-        return fail(DL_ENOMEM, "clover allocation failed");
-    const int grid = (int)std::max<long>(1, std::min<long>(((long)n + 255) / 256, (long)c->num_sms * 8));
-    CK(launch_ff_cast(reinterpret_cast<double *>(c->d_clov64), reinterpret_cast<double *>(c->d_clovff), n, 1, grid, c->cur));
-    CK(launch_ff_cast(reinterpret_cast<double *>(c->d_clovinv64), reinterpret_cast<double *>(c->d_clovff) + 2 * n, n, 1, grid,
-                      c->cur));
-    c->kernel_launches += 2;
-    c->clovff_ok = true;
-    return DL_OK;
-}
-// out = mat in (+ add) in float-float arithmetic on the half field of parity p, mat = A or (inv) A^-1.
-static int clover_mul_ff(dl_ctx *c, bool inv, int p, int N, const double *in, const double *add, double *out, bool ff) {
-    const long items = c->Vh * 2L * N;
-    const int grid = (int)std::max<long>(1, std::min<long>((items + 255) / 256, (long)c->num_sms * 8));
-    CK(launch_clover_mul_ff(c->d_clovff + (inv ? (size_t)c->V * 288 : 0), p, (int)c->Vh, N, in, add, out, ff, grid, c->cur));
-    c->kernel_launches++;
     return DL_OK;
 }
 
@@ -1275,20 +1249,12 @@ static int ff_cast(dl_ctx *c, const double *src, double *dst, size_t n_complex, 
 // the next cycle and the full-lattice residual; the final solution needs no
 // further hop.  op = P_DFF: b_o is float-float, x_o is left float-float and x_e
 // is first copied to float-float in c->bh64.
-// Clover: x_o = t + kappa A_oo^-1 D_oe x_e with t = A_oo^-1 b_o held in c->t64 (float-float
-// for op = P_DFF), and r = b_e - A_ee x_e + kappa D_eo x_o with A_ee x_e formed in c->bh64.
+// Clover (op = P_F64): x_o = t + kappa A_oo^-1 D_oe x_e with t = A_oo^-1 b_o held in
+// c->t64, and r = b_e - A_ee x_e + kappa D_eo x_o with A_ee x_e formed in c->bh64.
 static int outer_residual(dl_ctx *c, int op, int N, const double *be, const double *bo, const double *xe,
                           double *xo, double2 *pa, int *nb) {
     const double k = c->kappa;
     const int Vh = (int)c->Vh;
-    if (c->csw != 0.0 && op == P_DFF) {
-        TRY(ff_cast(c, xe, c->bh64, half_elems(c, N), 1));
-        TRY(do_hop(c, op, MODE_PLAIN, RED_NONE, xo, c->bh64, nullptr, nullptr, nullptr, 1, N, k, 0, Vh, nullptr, nullptr,
-                   FF_OUT));
-        TRY(clover_mul_ff(c, true, 1, N, xo, c->t64, xo, true));
-        TRY(clover_mul_ff(c, false, 0, N, c->bh64, nullptr, c->bh64, true));
-        return do_hop(c, op, MODE_RESID, RED_NORM, c->r64, xo, c->bh64, be, nullptr, 0, N, -k, 0, Vh, pa, nb, FF_Y);
-    }
     if (c->csw != 0.0) {
         TRY(do_hop(c, P_F64, MODE_XPAY, RED_NONE, xo, xe, c->t64, nullptr, nullptr, 1, N, k, 0, Vh, nullptr, nullptr,
                    0, nullptr, true));
@@ -1387,7 +1353,7 @@ static int solve_batch(dl_ctx *c, int n, int N, const SolveCfg &P, std::vector<O
     const bool clov = c->csw != 0.0;
     if (clov && P.method == DL_METHOD_CGNR)  // A_ee^-1 Mhat is not gamma_5-hermitian: CGNR's gamma_5 trick fails
         return fail(DL_EINVAL, "the clover operator is solved with BiCGStab only");
-    const int op = (P.prec != P_F64 && P.outer_dff && P.tol >= kFFMinTol) ? P_DFF : P_F64;
+    const int op = (!clov && P.prec != P_F64 && P.outer_dff && P.tol >= kFFMinTol) ? P_DFF : P_F64;
     const bool ffo = op == P_DFF;
     const int Vh = (int)c->Vh;
     const size_t half = half_elems(c, N) * 2;  // doubles
@@ -1420,8 +1386,7 @@ static int solve_batch(dl_ctx *c, int n, int N, const SolveCfg &P, std::vector<O
     }
     // bhat = b_e + kappa D_eo b_o, |bhat|^2 (clover: b_o replaced by t = A_oo^-1 b_o, kept in c->t64)
     if (ffo) TRY(ff_cast(c, bo, bo, half / 2, 1));
-    if (clov && ffo) TRY(ensure_clover_ff(c));
-    if (clov) TRY(ffo ? clover_mul_ff(c, true, 1, N, bo, nullptr, c->t64, true) : clover_mul(c, c->d_clovinv64, 1, N, bo, c->t64));
+    if (clov) TRY(clover_mul(c, c->d_clovinv64, 1, N, bo, c->t64));
     TRY(do_hop(c, op, MODE_XPAY, RED_NORM, c->bh64, clov ? c->t64 : bo, be, nullptr, nullptr, 0, N, k, 0, Vh, pa, &nb));
     outer_update_kernel<<<N, kScalarThreads, 0, c->stream>>>(c->d_outer, c->d_rhs, pa, nb, N, 0, P.tol, P.max_outer, P.max_iter);
     c->kernel_launches++;
@@ -1472,9 +1437,7 @@ static int solve_batch(dl_ctx *c, int n, int N, const SolveCfg &P, std::vector<O
             c->kernel_launches += 3;
         } else {
             // clover: the inner system is A_ee^-1 Mhat, its source A_ee^-1 r (in c->bh64)
-            if (clov)
-                TRY(ffo ? clover_mul_ff(c, true, 0, N, c->r64, nullptr, c->bh64, false)
-                        : clover_mul(c, c->d_clovinv64, 0, N, c->r64, c->bh64));
+            if (clov) TRY(clover_mul(c, c->d_clovinv64, 0, N, c->r64, c->bh64));
             VecLaunch v = vec_launch(c, prec, N, 2 * (prec == P_F64 ? 16 : 8));
             CK(launch_inner_init(v, c->d_outer, c->d_rhs, clov ? c->bh64 : c->r64, lo_ptr(c, LX), lo_ptr(c, LR),
                                  lo_ptr(c, LRH), lo_ptr(c, LP), pa, (cycle == 0 || P.restart) ? 1 : 0));

@@ -165,62 +165,6 @@ static __global__ void clover_mul_kernel(const double2 *mat, int p, int Vh, int 
     }
 }
 
-// out = mat x in (ADD: add + mat x in) in float-float arithmetic, mat a float-float
-// copy of A or A^-1; one thread per (site, block, right-hand side), out may equal in.
-// FF: in and out (and add) are float-float fields, else FP64 ones.  Bound by the FP32
-// units, 1700 instructions a thread against 288 FP64 ones (16^3 x 32, width 32: 275
-// us, in FP64 988 us).
-template <bool FF, bool ADD>
-static __global__ void __launch_bounds__(256) clover_mul_ff_kernel(const float4 *mat, int p, int Vh, int N, const double2 *in,
-                                                                   const double2 *add, double2 *out) {
-    typedef cx<dfloat> cff;
-    auto load = [](const double2 *f) {
-        const double2 v = *f;
-        if (FF) {
-            const float4 w = make_float4(__int_as_float(__double2loint(v.x)), __int_as_float(__double2hiint(v.x)),
-                                         __int_as_float(__double2loint(v.y)), __int_as_float(__double2hiint(v.y)));
-            return mk(dfloat(w.x, w.y), dfloat(w.z, w.w));
-        }
-        return mk(df_from_bits((uint32_t)__double2loint(v.x), (uint32_t)__double2hiint(v.x)),
-                  df_from_bits((uint32_t)__double2loint(v.y), (uint32_t)__double2hiint(v.y)));
-    };
-    const long total = (long)Vh * 2 * N;
-    for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-        const int r = (int)(idx % N);
-        const int b = (int)((idx / N) % 2);
-        const long cb = idx / (2L * N);
-        const float4 *m = mat + ((size_t)p * Vh + cb) * 72 + b * 36;
-        cff v[6];
-#pragma unroll
-        for (int j = 0; j < 6; ++j) v[j] = load(in + (cb * 12 + 6 * b + j) * (size_t)N + r);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            cdacc o = cda_zero();
-#pragma unroll
-            for (int j = 0; j < 6; ++j) {
-                const float4 w = __ldg(m + i * 6 + j);
-                cda_mac<false>(o, mk(dfloat(w.x, w.y), dfloat(w.z, w.w)), v[j]);
-            }
-            cff z = mk(da_norm(o.re), da_norm(o.im));
-            const size_t k = (cb * 12 + 6 * b + i) * (size_t)N + r;
-            if (ADD) z = load(add + k) + z;
-            if (FF) reinterpret_cast<float4 *>(out)[k] = make_float4(z.re.hi, z.re.lo, z.im.hi, z.im.lo);
-            else out[k] = make_double2(df_to_f64(z.re), df_to_f64(z.im));
-        }
-    }
-}
-
-cudaError_t launch_clover_mul_ff(const float *mat, int p, int Vh, int N, const double *in, const double *add, double *out,
-                                 bool ff, int grid, cudaStream_t s) {
-    const float4 *m = reinterpret_cast<const float4 *>(mat);
-    const double2 *i = reinterpret_cast<const double2 *>(in), *a = reinterpret_cast<const double2 *>(add);
-    double2 *o = reinterpret_cast<double2 *>(out);
-    if (ff && add) clover_mul_ff_kernel<true, true><<<grid, 256, 0, s>>>(m, p, Vh, N, i, a, o);
-    else if (ff) clover_mul_ff_kernel<true, false><<<grid, 256, 0, s>>>(m, p, Vh, N, i, a, o);
-    else clover_mul_ff_kernel<false, false><<<grid, 256, 0, s>>>(m, p, Vh, N, i, a, o);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_clover_build(const double *g64, const Geom &g, const SigmaBlocks &sig, double kcsw, double2 *a64,
                                double2 *ainv64, float2 *ainv32, __nv_bfloat162 *ainv16, int grid, cudaStream_t s) {
     clover_build_kernel<<<grid, 128, 0, s>>>(reinterpret_cast<const double2 *>(g64), g, sig, kcsw, a64, ainv64, ainv32,

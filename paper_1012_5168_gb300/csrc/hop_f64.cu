@@ -60,7 +60,6 @@ cudaError_t launch_hop_ff(int mode, int red, int fmt, const HopArgs &a, Launch &
 #define DL_CASE(m, rd, y, o) \
     if (mode == m && red == rd && yff == y && off == o) return go_ff<m, rd, y, o>(a, l);
     DL_CASE(MODE_PLAIN, RED_NONE, false, false)
-    DL_CASE(MODE_PLAIN, RED_NONE, false, true)
     DL_CASE(MODE_XPAY, RED_NONE, false, false)
     DL_CASE(MODE_XPAY, RED_NONE, true, false)
     DL_CASE(MODE_XPAY, RED_NONE, true, true)

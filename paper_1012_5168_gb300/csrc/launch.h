@@ -158,10 +158,6 @@ cudaError_t launch_resident_links(int prec, const double *g64, const uint32_t *c
 // out += acc_s (in - mat x in).
 cudaError_t launch_clover_build(const double *g64, const Geom &g, const SigmaBlocks &sig, double kcsw, double2 *a64,
                                double2 *ainv64, float2 *ainv32, __nv_bfloat162 *ainv16, int grid, cudaStream_t s);
-// The same product in float-float arithmetic with a float-float copy of the blocks; ff: the
-// fields are float-float (and out = add + mat x in for add != null), else FP64.
-cudaError_t launch_clover_mul_ff(const float *mat, int p, int Vh, int N, const double *in, const double *add, double *out,
-                                 bool ff, int grid, cudaStream_t s);
 cudaError_t launch_clover_mul(const double2 *mat, int p, int Vh, int N, const double *in, double *out, double acc_s,
                              int grid, cudaStream_t s);
 
