@@ -459,11 +459,14 @@ int dl_tune_hop(dl_ctx *ctx, int precision, int n_rhs, int force_R, int force_bl
  * (cls: 0 plain, 1 fused, 2 fused with the five BiCGStab reductions; see
  * dl_tune_hop) of width n_rhs in the inner storage for `precision`:
  * right-hand sides per thread, threads per block and kernel kind (outputs may
- * be NULL).  No tuning, no GPU work.  Errors: DL_EINVAL. */
+ * be NULL).  Inner phases that run in one launch, FP32 clover hops of width 32 and 16, and FP64 hops
+ * with at most 64 (site, right-hand side) items per SM take kernels of their own instead.  No
+ * tuning, no GPU work.  Errors: DL_EINVAL. */
 int dl_hop_shape(dl_ctx *ctx, int precision, int n_rhs, int cls, int *R_out, int *block_out, int *kind_out);
 /* Set that launch shape explicitly (R in {1, 2, 4}, block in {64, 128, 256},
- * kind 0-11 as dl_tune_hop; kinds 3-5, 9 and 11 take block 64 and size their own
- * blocks); the width then counts as tuned and pinned.  Errors: DL_EINVAL for a shape the
+ * kind as dl_tune_hop; kinds 3-5, 9 and 11 take block 64 and size their own
+ * blocks, kind 12 takes 128); the width then counts as tuned and pinned.  Every shape that
+ * dl_hop_shape reports is taken.  Errors: DL_EINVAL for a shape the
  * precision, width or storage layout does not allow. */
 int dl_set_hop_shape(dl_ctx *ctx, int precision, int n_rhs, int cls, int R, int block, int kind);
 

@@ -478,7 +478,7 @@ static int time_hops(dl_ctx *c, int prec, int N, int reps, float *ms_out, int wh
 // {64, 128, 256}).
 static bool shape_ok(int prec, int N, int R, int B, int bi, int pf) {
     if (pf < 0 || pf > 12 || (prec == P_F64 && (pf != 0 || R != 1))) return false;
-    if (pf == 12) return prec == P_F32 && R == 1 && N == 16 && bi == 0;
+    if (pf == 12) return prec == P_F32 && R == 1 && N == 16 && bi == 1;  // (its blocks have 128 threads)
     if (pf == 10 && (prec != P_F32 || R != 1)) return false;       // wider-cap direct: FP32, one per thread
     if (prec == P_F32P ? (pf != 0 && (pf < 7 || pf > 9)) : (pf >= 7 && pf <= 9)) return false;  // paired: 0, 7-9
     if (pf == 11 && prec == P_F32P) return false;
@@ -621,7 +621,7 @@ extern "C" int dl_set_hop_shape(dl_ctx *c, int precision, int n_rhs, int cls, in
         return fail(DL_EINVAL, "bad arguments");
     const int N = pow2_at_least(n_rhs), l = ilog2(N), ip = inner_prec(c, precision, N), m = cls;
     const int bi = block == 64 ? 0 : (block == 128 ? 1 : (block == 256 ? 2 : -1));
-    if ((R != 1 && R != 2 && R != 4) || bi < 0 || kind > 11 || !shape_ok(ip, N, R, block, bi, kind))
+    if ((R != 1 && R != 2 && R != 4) || bi < 0 || !shape_ok(ip, N, R, block, bi, kind))
         return fail(DL_EINVAL, "launch shape not available for this precision, width and layout");
     c->hop_R[ip][l][m] = R;
     c->hop_block[ip][l][m] = block;
@@ -742,7 +742,7 @@ extern "C" int dl_create(dl_ctx **out, const int dims[4], int t_bc, void *cuda_s
     for (int p = 0; p < 5; ++p)
         for (int l = 0; l < 8; ++l) {
             for (int m = 0; m < 3; ++m) {
-                c->hop_R[p][l][m] = 2;
+                c->hop_R[p][l][m] = p == P_F64 || l == 0 ? 1 : 2;
                 c->hop_block[p][l][m] = p == P_F64 ? 64 : 128;  // (FP64: the best or within 1% at every width)
                 c->hop_kind[p][l][m] = 0;
             }
