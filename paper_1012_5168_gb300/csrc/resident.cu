@@ -1,6 +1,4 @@
 // Launch of the cluster-resident solver (resident.cuh) and its link layout.
-#include <mutex>
-
 #include "launch.h"
 #include "resident.cuh"
 

@@ -1,8 +1,6 @@
 // Launch of one instantiation of the cluster-resident solver: n clusters of C blocks.
 #pragma once
 
-#include <mutex>
-
 #include "launch.h"
 #include "resident.cuh"
 
@@ -36,11 +34,10 @@ inline cudaError_t resident_opt_in(K kernel, size_t smem) {
 // Clusters of C blocks that can be resident at once (0: size not available).
 template <typename K>
 inline int resident_max_clusters(K kernel, size_t smem, int C) {
-    if (resident_opt_in(kernel, smem) != cudaSuccess) return 0;
     ResConfig c(C, 1, smem, 0);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &c.cfg) != cudaSuccess) {
-        cudaGetLastError();
+    if (resident_opt_in(kernel, smem) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, kernel, &c.cfg) != cudaSuccess) {
+        cudaGetLastError();  // (an answer, not a failure: the solve goes step by step)
         return 0;
     }
     return n;
