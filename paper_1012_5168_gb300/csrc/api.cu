@@ -1276,17 +1276,20 @@ static int outer_residual(dl_ctx *c, int op, int N, const double *be, const doub
 // a ragged batch maps its right-hand sides as a full one does.  C: the smallest
 // cluster that gives every SM at most one round of sites, or the largest of which
 // N are resident at once (more clusters than fit run in waves).
-// The line.  An iteration of the resident kernel takes about 8 + 11 us per round
-// of 128 sites per SM, one of the step-by-step iteration 36 us (its eight
-// launches) + 0.5 us per 1000 (site, right-hand side) pairs.  Measured (GB300,
-// FP32 unless said, resident against step by step, a solve): 4^4, 64 right-hand
-// sides 0.72 / 1.39 ms; 4^2 x 6 x 8, 12: 1.40 / 3.18; 6 x 10 x 4 x 12 BF16, 5:
-// 2.9 / 5.4; 6^3 x 8, 32: 2.1 / 3.5; 8^3 x 16: 1: 2.5 / 3.6, 8: 4.1 / 5.1, 32: 8.6 /
-// 9.1; beyond the line 8^3 x 16, 16: 7.2 / 5.9; 12^3 x 16, 4: 7.2 / 7.3, 1: 6.3 /
-// 4.8; 12^3 x 24, 2: 10.8 / 7.9.  FP64 is bound by the FP64 units (30 / 16 ms on
-// 8^3 x 16) and the clover term's site matrices do not suit the layout (3.3 / 2.5):
-// both stay step by step, as do timed hops, pinned launch shapes, continued cycles
-// and the paired layout.
+// The line, at most 3 + Vh N / 23000 rounds of 128 sites per SM and at most 8, errs
+// towards step by step.  Measured (GB300, N sources, kappa 0.125): the time of a
+// step-by-step solve over that of a resident one, FP32 / BF16 BiCGStab, FP32 / BF16 CGNR,
+//   N    last rounds within the line      beyond it
+//   1    3: 1.12 1.09, 1.20 1.16          4: 1.01 0.97, 1.03 0.96
+//   2    3: 1.23 1.23, 1.34 1.21          5: 1.08 0.91, 1.10 0.94
+//   4    4: 1.24 1.21, 1.23 1.11          6: 1.14 1.03, 1.15 0.97
+//   8    4: 1.19 1.22, 1.18 1.24          6: 1.08 1.09, 1.03 1.05;  8: 0.93 0.89, 0.88 0.87
+//   16   4: 1.18 1.15, 1.10 1.22          6: 1.03 1.10, 0.96 1.08;  8: 0.89 0.90, 0.85 0.91
+//   32   8: 1.19 1.15, 1.14 1.21          9: 1.09 1.09, 1.11 1.10
+//   64   8: 1.30 1.24, 1.25 1.25          10: 1.12 1.13, 1.18 1.16
+// FP64 is bound by the FP64 units (30 ms a solve on 8^3 x 16 against 16) and the clover
+// term's site matrices do not suit the layout (3.3 / 2.5): both stay step by step, as do
+// timed hops, pinned launch shapes, continued cycles and the paired layout.
 static bool resident_plan(dl_ctx *c, const SolveCfg &P, int N, int *C_out) {
     const int prec = P.prec;
     if (prec == P_F64 || c->csw != 0.0 || !P.restart || c->timing || c->hop_pinned[prec][ilog2(N)] ||
