@@ -1,8 +1,8 @@
 """A cluster size that the device refuses is answered with 0 clusters and leaves no CUDA error behind.
 
-The launch header is compiled into a small program, which asks for more shared memory than any SM has (on a
-machine without a GPU the request fails for that reason instead).  A later check of the last error must find
-none, or the solve that falls back to the step-by-step path would fail on it.
+The launch header is compiled into a small program, which asks for more shared memory than any SM has; the
+attribute call refuses that on the host.  A later check of the last error must find none, or the solve that
+falls back to the step-by-step path would fail on it (GPU: without one, every call reports that error).
 """
 
 import os
@@ -12,6 +12,8 @@ import subprocess
 import pytest
 
 from paper_1012_5168_gb300 import build
+
+pytestmark = pytest.mark.gpu
 
 SOURCE = r"""
 #include <cstdio>
