@@ -2342,9 +2342,10 @@ extern "C" int dl_meson_correlators(dl_ctx *c, const void *prop, const int src[4
     TRY(ensure_scratch(c->s_msum, sizeof(FourierSum) * (size_t)T * m.n_rep * MESON_E));
     TRY(ensure_scratch(c->s_out, sizeof(double2) * (size_t)n_mom * 256 * T));
     const size_t smem = 144 * 33 * sizeof(double2);
-    CK(cudaFuncSetAttribute(meson_site_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    meson_site_kernel<<<(int)((c->V + 31) / 32), 320, smem, c->stream>>>((const double2 *)prop, (int)c->V, V3,
-                                                                        (double2 *)c->s_site.p);
+    auto site_kernel = (uintptr_t)prop % 16 ? meson_site_kernel<false> : meson_site_kernel<true>;
+    CK(cudaFuncSetAttribute(site_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    site_kernel<<<(int)((c->V + 31) / 32), 320, smem, c->stream>>>((const double *)prop, (int)c->V, V3,
+                                                                  (double2 *)c->s_site.p);
     const long rows = (long)T * MESON_E;
     fourier_kernel<2><<<dim3((unsigned)((rows + 7) / 8), (m.n_rep + 3) / 4), 128, 0, c->stream>>>(
         (const double2 *)c->s_site.p, m.phase, m.zero, V3, rows, m.n_rep, (FourierSum *)c->s_msum.p);

@@ -311,12 +311,18 @@ __host__ __device__ __forceinline__ int meson_entry(int be, int al, int be2, int
 // lane per site.  Bound by FP64 (4896 FMA a site, 1.0 ms on 16^3 x 32; all 256
 // entries took 1.95 ms): the hermitian half is all that is formed, and stored
 // entry-major so that lanes write, and the Fourier sums read, contiguous sites.
-static __global__ void __launch_bounds__(320) meson_site_kernel(const double2 *prop, int V, int V3, double2 *out) {
+// prop may lie on any 8-byte boundary: one that is not a 16-byte boundary (AL16 false) is
+// read a double at a time.
+template <bool AL16>
+static __global__ void __launch_bounds__(320) meson_site_kernel(const double *prop, int V, int V3, double2 *out) {
     extern __shared__ double2 msm[];  // [144][33]
     const int s0 = blockIdx.x * 32, ns = min(32, V - s0);
     for (int k = threadIdx.x; k < 12 * 384; k += 320) {
         const int col = k / 384, e = k - col * 384, site = e / 12, c = e - site * 12;
-        if (site < ns) msm[(col * 12 + c) * 33 + site] = __ldg(prop + ((size_t)col * V + s0) * 12 + e);
+        const double *v = prop + (((size_t)col * V + s0) * 12 + e) * 2;
+        if (site < ns)
+            msm[(col * 12 + c) * 33 + site] =
+                AL16 ? __ldg(reinterpret_cast<const double2 *>(v)) : make_double2(__ldg(v), __ldg(v + 1));
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
