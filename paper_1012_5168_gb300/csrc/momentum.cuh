@@ -110,12 +110,14 @@ static __global__ void group_site_kernel(double2 *site, long per, int ng, int gr
 // w >> 2; a lane for (site, beta), so the three products of a colour are one
 // warp-wide decision: where a diluted eta vanishes for the whole warp the FP64
 // work is left out (dense fields are bound by FP64: 192 FMA a site and pair, 1.2 ms
-// for 48 pairs on 16^3 x 32; diluted ones by reading the fields, 0.36 ms), except
+// for 48 pairs on 16^3 x 32; diluted ones by shared memory, 0.65 ms, where reading the
+// fields takes 0.36: all warps read f for every colour, and sites lie 384 bytes apart), except
 // that a non-finite phi still makes the sum NaN, as 0 times it would.
 struct CanonSpinArgs {
     const double2 *eta, *phi;  // canonical [n][V][12]
     Geom g;
-    int V3, group, nt;         // nt timeslices from 0, or (tgrp) one timeslice per group
+    int V3, group, nt;         // pairs per block; nt timeslices from 0, or (tgrp) one timeslice per group
+    int parts;                 // blocks that share a group's pairs: gridDim.z = groups x parts = slots of out
     const int *tgrp;
     double2 *out;
 };
@@ -129,7 +131,7 @@ __device__ __forceinline__ bool cx_bad(double2 z) {  // infinite or NaN, without
 static __global__ void __launch_bounds__(256) canon_spin_kernel(CanonSpinArgs A) {
     __shared__ double2 se[2][384], sf[2][384];
     const int tile = blockIdx.x, tt = blockIdx.y, gi = blockIdx.z;
-    const int t = A.tgrp ? A.tgrp[gi] : tt;
+    const int t = A.tgrp ? A.tgrp[gi / A.parts] : tt;
     const int s0 = tile * 32, ns = min(32, A.V3 - s0);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, al = w & 3, par = w >> 2, be = lane & 3;
     const long V = (long)A.V3 * A.g.L[3];
@@ -200,67 +202,57 @@ struct __align__(16) FourierSum {
 // real sums
 //   out[row][r] = (sum c x, sum s y, sum c y, sum s x)   of  z = x + i y = in[row][site]
 // give the sums of z and of conj(z) at p and at -p.  in: [rows][V3] (a row is one
-// matrix entry on one timeslice).  A warp takes EPW rows and up to four
-// representatives (blockIdx.y picks which): its lanes walk the sites (coalesced,
-// each phase used for EPW rows), and the lane sums meet in a fixed order.  A
-// representative with zero momentum (zero[r]) needs sums of x and y only.
-template <int EPW>
+// matrix entry on one timeslice).  A warp takes a row and up to four representatives
+// (blockIdx.y picks which): its lanes walk the sites (coalesced).  At the end the lanes
+// exchange halves of their 16 sums instead of each adding all of them, 16 FP64
+// additions a warp instead of 80.  Bound by FP64: 3072 rows and 172 representatives of 4096 sites
+// are 13.9 ms of FMA, and the loops of 24 pairs that ask for them take 15.1 ms.  (Two rows a
+// warp, each phase loaded once for both: slower.)  A lone representative of zero momentum (zero[r0])
+// needs sums of x and y only; among others its phases are ones and zeros like any: told apart in
+// the loop, the compiler issued both kinds of sums, half as many FP64 instructions again (23.9 ms).
 static __global__ void __launch_bounds__(128) fourier_kernel(const double2 *in, const double2 *ph, const int *zero,
                                                              int V3, long rows, int n_rep, FourierSum *out) {
     const int lane = threadIdx.x & 31;
-    const long row = ((long)blockIdx.x * 4 + (threadIdx.x >> 5)) * EPW;
+    const long row = (long)blockIdx.x * 4 + (threadIdx.x >> 5);
     const int r0 = blockIdx.y * 4;
     if (row >= rows) return;
-    FourierSum acc[EPW][4];
-    bool z[4];
+    double acc[16];  // [4 representative + sum]
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        z[r] = r0 + r < n_rep && zero[r0 + r] != 0;
+    for (int k = 0; k < 16; ++k) acc[k] = 0.0;
+    const double2 *src = in + (size_t)row * V3;
+    if (n_rep - r0 == 1 && zero[r0]) {
+        for (int s = lane; s < V3; s += 32) {
+            const double2 v = __ldg(src + s);
+            acc[0] += v.x;
+            acc[2] += v.y;
+        }
+    } else {
+        const double2 *w_[4];
 #pragma unroll
-        for (int e = 0; e < EPW; ++e) acc[e][r] = FourierSum{0.0, 0.0, 0.0, 0.0};
-    }
-    for (int s = lane; s < V3; s += 32) {
-        double2 v[EPW];
+        for (int r = 0; r < 4; ++r) w_[r] = ph + (size_t)min(r0 + r, n_rep - 1) * V3;
+        for (int s = lane; s < V3; s += 32) {
+            const double2 v = __ldg(src + s);
 #pragma unroll
-        for (int e = 0; e < EPW; ++e) v[e] = row + e < rows ? __ldg(in + (size_t)(row + e) * V3 + s) : make_double2(0.0, 0.0);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            if (r0 + r >= n_rep) break;
-            if (z[r]) {
-#pragma unroll
-                for (int e = 0; e < EPW; ++e) {
-                    acc[e][r].x += v[e].x;
-                    acc[e][r].z += v[e].y;
-                }
-            } else {
-                const double2 w = __ldg(ph + (size_t)(r0 + r) * V3 + s);
-#pragma unroll
-                for (int e = 0; e < EPW; ++e) {
-                    acc[e][r].x = ::fma(w.x, v[e].x, acc[e][r].x);
-                    acc[e][r].y = ::fma(w.y, v[e].y, acc[e][r].y);
-                    acc[e][r].z = ::fma(w.x, v[e].y, acc[e][r].z);
-                    acc[e][r].w = ::fma(w.y, v[e].x, acc[e][r].w);
-                }
+            for (int r = 0; r < 4; ++r) {
+                if (r0 + r >= n_rep) break;
+                const double2 w = __ldg(w_[r] + s);
+                acc[4 * r] = ::fma(w.x, v.x, acc[4 * r]);
+                acc[4 * r + 1] = ::fma(w.y, v.y, acc[4 * r + 1]);
+                acc[4 * r + 2] = ::fma(w.x, v.y, acc[4 * r + 2]);
+                acc[4 * r + 3] = ::fma(w.y, v.x, acc[4 * r + 3]);
             }
         }
     }
 #pragma unroll
-    for (int e = 0; e < EPW; ++e)
+    for (int h = 8; h >= 1; h >>= 1) {  // the lanes with bit 2 h set keep the upper h sums
+        const bool up = (lane & (2 * h)) != 0;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            if (r0 + r >= n_rep) break;
-            FourierSum &a = acc[e][r];
-#pragma unroll
-            for (int off = 16; off >= 1; off >>= 1) {
-                a.x += __shfl_xor_sync(0xffffffffu, a.x, off);
-                a.z += __shfl_xor_sync(0xffffffffu, a.z, off);
-                if (!z[r]) {
-                    a.y += __shfl_xor_sync(0xffffffffu, a.y, off);
-                    a.w += __shfl_xor_sync(0xffffffffu, a.w, off);
-                }
-            }
-            if (lane == 0 && row + e < rows) out[(size_t)(row + e) * n_rep + r0 + r] = a;
-        }
+        for (int k = 0; k < h; ++k)
+            acc[k] = (up ? acc[h + k] : acc[k]) + __shfl_xor_sync(0xffffffffu, up ? acc[k] : acc[h + k], 2 * h);
+    }
+    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+    const int k = lane >> 1;  // the sum that this lane holds
+    if ((lane & 1) == 0 && r0 + (k >> 2) < n_rep) reinterpret_cast<double *>(out + (size_t)row * n_rep + r0)[k] = acc[0];
 }
 // sum of e^{-i p.x} z (CONJ: of e^{-i p.x} conj(z)) from the four sums; sg = -1: at -p.
 template <bool CONJ> __device__ __forceinline__ double2 fourier_value(FourierSum f, int sg) {
