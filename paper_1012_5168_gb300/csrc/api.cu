@@ -180,6 +180,13 @@ static Launch make_launch(dl_ctx *c, long items, int block, size_t smem, int per
     return l;
 }
 
+// Whether pairs come in runs of twelve or more on one timeslice, as sources diluted in time, spin and colour do.
+static bool in_runs(const int *t, int n) {
+    int runs = 1;
+    for (int j = 1; j < n; ++j) runs += t[j] != t[j - 1];
+    return 12 * runs <= n;
+}
+
 static size_t half_elems(dl_ctx *c, int N) { return (size_t)c->Vh * 12 * N; }  // complex per half field
 
 static int storage_bytes(int prec) {
@@ -1741,9 +1748,10 @@ extern "C" int dl_apply_clover(dl_ctx *c, const void *in, void *out, int n_rhs, 
 // buffer holding the result (ping-pong with `spare`).
 // Smear *buf (and, if buf2 is set, *buf2 in the same launches) in place over the cb
 // range; spare / spare2 are scratch fields of the same shape.  On return *buf
-// (*buf2) points at whichever of the pair holds the result.
+// (*buf2) points at whichever of the pair holds the result.  diluted: the fields may
+// well have spins that vanish (the result is the same either way).
 static int smear_eo(dl_ctx *c, double **buf, double *spare, int N, int n, const dl_smear &s, int cb0, int cb1,
-                    const int *tcol = nullptr, double **buf2 = nullptr, double *spare2 = nullptr) {
+                    const int *tcol = nullptr, double **buf2 = nullptr, double *spare2 = nullptr, bool diluted = false) {
     if (buf2 && c->smear_fp64) {  // the FP64 kernel smears one field per launch
         TRY(smear_eo(c, buf, spare, N, n, s, cb0, cb1, tcol));
         return smear_eo(c, buf2, spare2, N, n, s, cb0, cb1, tcol);
@@ -1774,12 +1782,14 @@ static int smear_eo(dl_ctx *c, double **buf, double *spare, int N, int n, const 
     } else {
         double *src2 = buf2 ? *buf2 : nullptr, *dst2 = spare2;
         const int nf = buf2 ? 2 : 1;
-        // Where the dense groups (the four spins of a right-hand side) give no SM a second block,
-        // leaving out zero spins gains nothing, and finding them costs three launches' latency and a step's
-        // threads one more dependent load: 4 x 4 x 6, 24 pairs: 668 us without a list, 698 with one;
-        // 4 x 22 x 4 (198 blocks): 926 and 757.
+        // Leaving out zero spins gains nothing where the dense groups (the four spins of a right-hand side)
+        // give no SM a second block, and finding them costs a few launches and a step's threads two
+        // dependent loads more: 4 x 4 x 6, 24 pairs: 668 us without a list, 698 with one; 4 x 22 x 4 (198 blocks):
+        // 912 and 739.  Dense fields lose up to a tenth by that, and pairs on many timeslices a quarter
+        // (24 on 24 timeslices of 16^3: 7.9 and 10.9 ms; a list has both fields' groups in a block,
+        // which then holds fewer neighbouring sites).  So the caller says whether to look.
         Launch lr = make_launch(c, 2L * (cb1 - cb0) * 3 * n * nf, 256, 0, 64);
-        SmearList *L = lr.grid > c->num_sms ? c->d_smear : nullptr;
+        SmearList *L = diluted && lr.grid > c->num_sms ? c->d_smear : nullptr;
         Launch lc = make_launch(c, 2L * (cb1 - cb0) * 12 * n, 256, 0, 8);
         if (L) {
             Launch lf = make_launch(c, 2L * (cb1 - cb0) * n, 256, 0, 8);
@@ -1794,7 +1804,8 @@ static int smear_eo(dl_ctx *c, double **buf, double *spare, int N, int n, const 
         // one thread per (site, colour row, group of columns), sized for dense fields; the list's
         // length is known on the device only.  A grid that is resident at once (two blocks per SM)
         // spreads the list over all SMs: 22 x 6 x 4 (297 blocks), 24 pairs, 918 us; 971 without a
-        // list, 979 to 1009 with the list in the first blocks.
+        // list, 979 to 1009 with the list in the first blocks.  Dense fields lose little there (8^3, 24
+        // pairs, 50 steps: 1.03 ms both ways): the step sees that the list is full.
         const bool spread = L && lr.grid <= 2 * c->num_sms;
         if (spread) lr.grid = 2 * c->num_sms;
         for (int it = 0; it < s.n_iter; ++it) {
@@ -1802,9 +1813,11 @@ static int smear_eo(dl_ctx *c, double **buf, double *spare, int N, int n, const 
             A.out = dst;
             A.in2 = src2;
             A.out2 = dst2;
-            auto step = !L ? smear_ff_rows_kernel<false, false>
-                           : (spread ? smear_ff_rows_kernel<true, true> : smear_ff_rows_kernel<true, false>);
-            step<<<lr.grid, lr.block, 0, c->cur>>>(A, c->d_gauge_ff, L, nf);
+            if (!L)  // a field per grid row
+                smear_ff_rows_kernel<false, false><<<dim3((lr.grid + nf - 1) / nf, nf), lr.block, 0, c->cur>>>(
+                    A, c->d_gauge_ff, nullptr);
+            else if (spread) smear_ff_rows_kernel<true, true><<<lr.grid, lr.block, 0, c->cur>>>(A, c->d_gauge_ff, L);
+            else smear_ff_rows_kernel<true, false><<<lr.grid, lr.block, 0, c->cur>>>(A, c->d_gauge_ff, L);
             std::swap(src, dst);
             std::swap(src2, dst2);
         }
@@ -2055,7 +2068,7 @@ static int contract_mom_canon(dl_ctx *c, const double *eta, const double *phi, i
 // sinks into c->d_loops[j][sink][16][T] (or, with a MomSpec, into
 // mom->dst[sink][j][q][16][T]); smearing overwrites the buffers.
 static int trace_eo(dl_ctx *c, double *eta_buf, double *phi_buf, int n, int N, int sink, const dl_smear *sm, int t_lo,
-                    int t_hi, int n_sinks, const int *tcol = nullptr, const MomSpec *mom = nullptr) {
+                    int t_hi, int n_sinks, const int *tcol = nullptr, const MomSpec *mom = nullptr, bool diluted = false) {
     const int T = c->dims[3];
     const int cb0 = t_lo * c->g.V3h, cb1 = t_hi * c->g.V3h;
     const int per = 16 * T;
@@ -2068,7 +2081,7 @@ static int trace_eo(dl_ctx *c, double *eta_buf, double *phi_buf, int n, int N, i
         if (flag == DL_SINK_SMEARED) {
             const int s0 = tcol ? 0 : cb0, s1 = tcol ? c->g.V3h : cb1;
             TRY(smear_eo(c, &e, e == c->b64 ? c->s64a : c->b64, N, n, *sm, s0, s1, tcol, &f,
-                         f == c->x64 ? c->s64b : c->x64));
+                         f == c->x64 ? c->s64b : c->x64, diluted));
         }
         // contract into the slot `slot` region of d_loops viewed as [sink][n][16][T]
         if (mom)
@@ -2163,7 +2176,8 @@ extern "C" int dl_trace_loops(dl_ctx *c, const void *eta, const void *phi, int n
         }
         TRY(canon_to_eo(c, (const double *)eta + j0 * field, c->b64, n, N, 0, cb0, cb1, tcol));
         TRY(canon_to_eo(c, (const double *)phi + j0 * field, c->x64, n, N, 0, cb0, cb1, tcol));
-        TRY(trace_eo(c, c->b64, c->x64, n, N, sink, sm, t_lo, t_hi, n_sinks, tcol));
+        TRY(trace_eo(c, c->b64, c->x64, n, N, sink, sm, t_lo, t_hi, n_sinks, tcol, nullptr,
+                     tcol && in_runs(t_of_rhs + j0, n)));
         if (group <= 64) {
             const int ng = n / group;
             group_sum_kernel<<<std::max(1, (ng * n_sinks * per + 255) / 256), 256, 0, c->stream>>>(
@@ -2333,7 +2347,7 @@ extern "C" int dl_trace_loops_mom(dl_ctx *c, const void *eta, const void *phi, i
             TRY(canon_to_eo(c, f, c->x64, n, N, 0, cb0, cb1, tcol));
             MomSpec ms = m;
             ms.dst = m.dst + (local ? (size_t)N * per : 0);
-            TRY(trace_eo(c, c->b64, c->x64, n, N, DL_SINK_SMEARED, sm, 0, T, 1, tcol, &ms));
+            TRY(trace_eo(c, c->b64, c->x64, n, N, DL_SINK_SMEARED, sm, 0, T, 1, tcol, &ms, tcol && in_runs(ts, n)));
         }
         const int ng = n / group;
         group_sum_kernel<<<std::max(1, (ng * n_sinks * per + 255) / 256), 256, 0, c->stream>>>(
@@ -2466,7 +2480,7 @@ extern "C" int dl_exact_loops(dl_ctx *c, int64_t src_first, int64_t n_src, const
             const long V3 = 2L * c->g.V3h;
             const int ta = (int)((s0 / 12) / V3), tb = (int)(((s0 + n - 1) / 12) / V3) + 1;
             TRY(canon_to_eo(c, c->d_canon, c->b64, n, N, 0, ta * c->g.V3h, tb * c->g.V3h));
-            TRY(trace_eo(c, c->b64, c->x64, n, N, DL_SINK_SMEARED, sm, ta, tb, 1));
+            TRY(trace_eo(c, c->b64, c->x64, n, N, DL_SINK_SMEARED, sm, ta, tb, 1, nullptr, nullptr, true));
             sum_loops_kernel<<<std::max(1, (per + 255) / 256), 256, 0, c->stream>>>(c->d_loops, n, per, c->d_loops, per);
             add_kernel<<<std::max(1, (per + 255) / 256), 256, 0, c->stream>>>(accSm, c->d_loops, per);
             c->kernel_launches += 2;
@@ -2608,14 +2622,16 @@ static int tsm_pass(dl_ctx *c, uint64_t seed, int64_t first, int count, unsigned
         // eta: re-convert the sources (b64 was consumed by the solver).  Time-diluted
         // sources are contracted (and smeared) on their own timeslice only.
         const int *tcol = nullptr;
+        bool diluted = (dil & DL_DIL_SPIN) != 0;
         if (dil & DL_DIL_TIME) {
             int ts[64];
             for (int j = 0; j < n; ++j) ts[j] = t0 >= 0 ? t0 : (int)((first + (r0 + j) / K) % T);
             CK(cudaMemcpyAsync(c->d_tcol, ts, n * sizeof(int), cudaMemcpyHostToDevice, c->stream));
             tcol = c->d_tcol;
+            diluted = diluted && in_runs(ts, n);
         }
         TRY(canon_to_eo(c, c->d_canon, c->b64, n, N, 0, 0, tcol ? c->g.V3h : (int)c->Vh, tcol));
-        TRY(trace_eo(c, c->b64, c->x64, n, N, sink, sm, 0, T, n_sinks, tcol));
+        TRY(trace_eo(c, c->b64, c->x64, n, N, sink, sm, 0, T, n_sinks, tcol, nullptr, diluted));
         fold_noise_kernel<<<std::max(1, (n_sinks * per + 255) / 256), 256, 0, c->stream>>>(c->d_loops, n, N, per,
                                                                                            n_sinks, K, r0, out, 0);
         c->kernel_launches++;

@@ -566,16 +566,17 @@ static __global__ void smear_list_kernel(SmearList *L, int n, int nf, const int 
 // thread) measured 9% faster than three (85).  48 pairs of spin-diluted sources
 // and solutions on one 16^3 timeslice: 114 us a step with the groups, 176 us
 // on all 384 columns.
-// Without a list (LIST false) the groups are the four spins of each right-hand side of nf fields.
+// Without a list (LIST false) the groups are the four spins of each right-hand side, a field per blockIdx.y.
 // SPREAD: the grid holds more threads than there is work, and all its blocks take an equal part.
 template <bool LIST, bool SPREAD>
 static __global__ void __launch_bounds__(256, 2) smear_ff_rows_kernel(SmearArgs A, const float *gauge_ff,
-                                                                      const SmearList *L, int nf) {
-    const int nsite = A.cb1 - A.cb0, ng = LIST ? L->n_groups : A.n * nf;
+                                                                      const SmearList *L) {
+    const int nsite = A.cb1 - A.cb0, ng = LIST ? L->n_groups : A.n;
     const long total = 2L * nsite * 3 * ng;
     const size_t half = (size_t)A.g.Vh * 12 * A.N * 2;
     const ff fa = df_from_double(A.a), fc = df_from_double(A.c);
-    const int per = SPREAD ? (int)((total + gridDim.x - 1) / gridDim.x + 31) & ~31 : blockDim.x;
+    const bool dense = SPREAD && ng == (A.in2 ? 2 : 1) * A.n;  // nothing vanishes: no further look at the list
+    const int per = SPREAD && !dense ? (int)((total + gridDim.x - 1) / gridDim.x + 31) & ~31 : blockDim.x;
     if (SPREAD && (int)threadIdx.x >= per) return;
     for (long idx = (long)blockIdx.x * per + threadIdx.x; idx < total; idx += (long)gridDim.x * per) {
         const int gi = (int)(idx % ng);
@@ -584,11 +585,11 @@ static __global__ void __launch_bounds__(256, 2) smear_ff_rows_kernel(SmearArgs 
         const int sp = (int)(rest / 3);
         const int p = sp / nsite;
         SmearGroup G;
-        if (LIST) {
+        if (LIST && !dense) {
             G = L->g[gi];
         } else {
-            const int j = gi % A.n;
-            G.field = gi / A.n;
+            G.field = SPREAD ? gi / A.n : blockIdx.y;
+            const int j = SPREAD ? gi % A.n : gi;
             G.t = A.tcol ? A.tcol[j] : 0;
 #pragma unroll
             for (int k = 0; k < 4; ++k) G.col[k] = j << 2 | k;
