@@ -126,6 +126,7 @@ struct dl_ctx {
         size_t cap = 0;
     };
     Scratch s_phase, s_site, s_msum, s_mloops, s_mgroup, s_mom, s_cover, s_out;
+    std::vector<int> mom_host;  // source of the upload into s_mom, which may still be under way on return
 
     SmearList *d_smear = nullptr;  // columns and groups of the current smearing
 
@@ -2261,7 +2262,8 @@ static int build_phases(dl_ctx *c, const int *momenta, int n_mom, int ox, int oy
         }
     }
     const int nr = (int)zero.size();
-    std::vector<int> all(reps);
+    std::vector<int> &all = c->mom_host;
+    all = reps;
     all.insert(all.end(), zero.begin(), zero.end());
     all.insert(all.end(), map.begin(), map.end());
     TRY(ensure_scratch(c->s_mom, sizeof(int) * all.size()));

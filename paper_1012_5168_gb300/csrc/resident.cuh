@@ -1,5 +1,5 @@
-// Cluster-resident Krylov solver: a whole inner phase (BiCGStab or CGNR) of a
-// mixed-precision or FP64 solve in one launch, for problems that live in L2.
+// Cluster-resident Krylov solver: a whole inner phase (BiCGStab or CGNR, FP32 or BF16
+// fields) of a mixed-precision solve in one launch, for problems that live in L2.
 //
 // On a small lattice the step-by-step iteration (eight launches: four hops,
 // two vector updates, two scalar kernels) is bound by launch gaps and by the

@@ -4,8 +4,11 @@ The paper's production ran independent inversions spread over GPU nodes
 (Acknowledgements: an 8-node Tesla cluster and NCSA Lincoln).  Every noise
 vector or point source is independent, so ranks take disjoint contiguous index
 ranges.  There is no data-path collective: each rank produces its own loops and
-a host-side merge adds them in rank order, which makes the result identical
-whatever the number of ranks.
+a host-side merge adds them in rank order, whichever rank is done first.  Another
+number of ranks cuts the batches elsewhere, and the kernels that solve a source
+follow the width of its batch (a last batch of half the width or less takes a
+narrower one): the results then agree to the solver's tolerance, and bit by bit
+where every source keeps its batch.
 """
 
 from __future__ import annotations
