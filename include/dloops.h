@@ -45,7 +45,7 @@
  *                             restarting (measured slower);
  *   DLOOPS_OUTER_DFF=0        defect-correction hops of mixed-precision solves in
  *                             FP64 instead of float-float arithmetic (float-float is
- *                             used only for tol >= 1e-11);
+ *                             used only for tol >= 1e-11 and without the clover term);
  *   DLOOPS_HOP_ARITH=dff      dl_apply_hop / dl_apply_m in float-float arithmetic.
  */
 #ifndef DLOOPS_H
@@ -72,7 +72,8 @@ typedef enum dl_status {
  * BiCGStab; F32 and BF16 keep spinors and links in that storage type with FP32
  * arithmetic inside a defect-correction loop on FP64 fields (solution
  * accumulation and final result in FP64; the true residual in float-float
- * arithmetic, about 48 significant bits, for tol >= 1e-11, else in FP64).
+ * arithmetic, about 48 significant bits, for tol >= 1e-11 without the clover
+ * term, else in FP64).
  * Sec. 2: the paper's inversions use mixed-precision CG/BiCGStab. */
 enum { DL_PREC_F64 = 0, DL_PREC_F32 = 1, DL_PREC_BF16 = 2 };
 

@@ -1358,7 +1358,7 @@ static int solve_batch(dl_ctx *c, int n, int N, const SolveCfg &P, std::vector<O
     const double k = c->kappa, k2 = k * k;
     // Defect-correction hops (bhat, residuals, reconstruction) in float-float
     // arithmetic for mixed-precision solves whose tolerance lies well above its
-    // rounding (~1e-14 relative), else in FP64.  In float-float, b_o and x_o are
+    // rounding (~1e-14 relative), else (and with the clover term) in FP64.  In float-float, b_o and x_o are
     // held as float-float fields until the batch ends and x_e is copied to that
     // format (into the bhat buffer, free once r = bhat) before each residual.
     const bool clov = c->csw != 0.0;
