@@ -29,7 +29,12 @@ static cudaError_t go(const HopArgs &a, Launch &l) {
     }
     // 168 registers let six blocks of 64 threads share an SM (about 180: five).  One right-hand
     // side on 16^3 x 32: 115 / 121 / 141 us (plain, <rhat, v>, five sums) against 124 / 131 / 152.
-    auto kernel = hop_kernel_cap<double, R, MODE, RED, 168>;
+    // Beyond one round the blocks with a second item lie on some SMs and not on others.  With 7.5 to
+    // 10.5 blocks an SM (of any residency) that leaves six at once behind five: 8.0 blocks, plain hop, 145
+    // against 125 us, 9.5 blocks 181 / 156, at 7.2 and 10.5 both alike; from two rounds on six are ahead
+    // by 4% (14.2 blocks) or behind by 5% (16.4) and mostly alike.
+    const bool five = l.block == 64 && 2L * l.grid > 15L * l.num_sms && 2L * l.grid <= 21L * l.num_sms;
+    auto kernel = five ? hop_kernel<double, R, MODE, RED> : hop_kernel_cap<double, R, MODE, RED, 168>;
     clamp_grid(l, resident_blocks(kernel, l.block, l.smem));
     kernel<<<l.grid, l.block, l.smem, l.stream>>>(a);
     return cudaGetLastError();
